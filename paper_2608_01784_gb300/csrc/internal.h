@@ -175,10 +175,10 @@ struct GroupRows {
 };
 cudaError_t launch_swiglu_simt(int dtype, const void* x, const void* w_gate_up,
                                int d, int inter, const GroupRows& g, void* act,
-                               uint32_t* err, cudaStream_t stream);
+                               int num_sms, cudaStream_t stream);
 cudaError_t launch_down_simt(int dtype, const void* act, const void* w_down,
                              int d, int inter, const GroupRows& g, void* y,
-                             uint32_t* err, cudaStream_t stream);
+                             int num_sms, cudaStream_t stream);
 
 // ---- experts: tcgen05 grouped GEMMs (experts_tc.cu) -----------------------
 struct TcGemmArgs {

@@ -532,14 +532,14 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
     rx::GroupRows dense{nullptr, nullptr, nullptr, nullptr, 1, T, T};
     if (simt) {
       if (up) {
-        RX_CUDA(rx::launch_swiglu_simt(dtype, xperm, w_gate_up, d, inter, grouped, amid, err, s));
+        RX_CUDA(rx::launch_swiglu_simt(dtype, xperm, w_gate_up, d, inter, grouped, amid, sms, s));
         if (shared_inter)
-          RX_CUDA(rx::launch_swiglu_simt(dtype, hidden, shared_gate_up, d, shared_inter, dense, ash, err, s));
+          RX_CUDA(rx::launch_swiglu_simt(dtype, hidden, shared_gate_up, d, shared_inter, dense, ash, sms, s));
       }
       if (down) {
-        RX_CUDA(rx::launch_down_simt(dtype, amid, w_down, d, inter, grouped, xperm, err, s));
+        RX_CUDA(rx::launch_down_simt(dtype, amid, w_down, d, inter, grouped, xperm, sms, s));
         if (shared_inter)
-          RX_CUDA(rx::launch_down_simt(dtype, ash, shared_down, d, shared_inter, dense, ysh, err, s));
+          RX_CUDA(rx::launch_down_simt(dtype, ash, shared_down, d, shared_inter, dense, ysh, sms, s));
       }
     } else {
       CUtensorMap ma1, mb1, ma2, mb2;
