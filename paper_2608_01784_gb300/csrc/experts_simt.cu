@@ -110,6 +110,13 @@ __device__ __forceinline__ f32x2 sub2(f32x2 a, f32x2 b) {  // a - b: -1 * b is e
   return fma2(b, pack2(-1.0f, -1.0f), a);
 }
 
+template <typename Te>
+__device__ __noinline__ float plain_dot(const Te* x, const Te* w, int K) {
+  float s = 0.f;
+  for (int k = 0; k < K; ++k) s = __fmaf_rn(to_f32(x[k]), to_f32(w[k]), s);
+  return s;
+}
+
 // Group of 128-row tile mt: the expert whose tile prefix holds it (a 32-ary
 // search, every warp for itself); -1 when there is none.
 __device__ __forceinline__ int group_of_tile(const GroupRows& g, int mt) {
@@ -225,10 +232,6 @@ __global__ void __launch_bounds__(C::NT, 1)
   };
 
   f32x2 acc2[TM][HN], run[TM][HN];  // pairs of adjacent columns: total, running sum
-#pragma unroll
-  for (int i = 0; i < TM; ++i)
-#pragma unroll
-    for (int j = 0; j < HN; ++j) acc2[i][j] = run[i][j] = 0ull;
   const int nkb = K / BK;
   // Block kb: its loads were issued two blocks ago (one block's fmas do not
   // cover an L2 miss), the next block's values go to the other buffer, which
@@ -279,6 +282,10 @@ __global__ void __launch_bounds__(C::NT, 1)
     if (kb + 1 < nkb) store(Other{});
     __syncthreads();
   };
+#pragma unroll
+  for (int i = 0; i < TM; ++i)
+#pragma unroll
+    for (int j = 0; j < HN; ++j) acc2[i][j] = run[i][j] = 0ull;
   load(0, Int<0>{});
   if (nkb > 1) load(BK, Int<1>{});
   store(Int<0>{});
@@ -315,6 +322,16 @@ __global__ void __launch_bounds__(C::NT, 1)
   for (int i = 0; i < TM; ++i) {
     const int r = ty * TM + i;
     if (r >= rows) continue;
+    // what rounds off an infinite sum is a NaN, so a NaN may stand for an
+    // infinity: such an output is summed again without the carry
+#pragma unroll
+    for (int j = 0; j < TN; ++j) {
+      const int c = n0 + tx * HN + (j % HN) + (MODE == 1 && j >= HN ? BN / 2 : 0);
+      if (acc[i][j] != acc[i][j] && c < n_total)
+        acc[i][j] = plain_dot(xe + static_cast<int64_t>(r) * K,
+                              we + (MODE == 0 && j >= HN ? static_cast<int64_t>(n_total) + c : c) *
+                                       static_cast<int64_t>(K), K);
+    }
     Te* orow = out + static_cast<int64_t>(row0 + r) * n_total;
     if (MODE == 0) {
       float v[HN];

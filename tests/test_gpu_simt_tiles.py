@@ -48,3 +48,20 @@ def test_tile_edges(dtype, T, E, kmax, d, inter, shared):
         assert rel <= G.F32_REL_L2 and mx <= G.F32_MAX_ABS, (rel, mx)
     else:
         assert rel <= G.BF16_REL_L2 and mx <= G.BF16_MAX_ABS, (rel, mx)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("T,inter", [(40, 64), (2500, 512)])
+def test_an_overflowing_sum_stays_infinite(T, inter):
+    # up weights of 1e38: every up sum of 64 ones is +inf, the gate sums are
+    # 64, so act = 64 * inf and y, with positive down weights, is +inf
+    d = 64
+    cfg, layer = _case("f32", T, 1, 1, d, inter, 0, seed=T)
+    layer["hidden"][:] = 1.0
+    layer["w_gate_up"][:, :inter] = 1.0
+    layer["w_gate_up"][:, inter:] = 1e38
+    layer["w_down"][:] = 1.0
+    gl = G.GpuLayer(cfg, layer)
+    out, _, status = gl.forward(np.ones(T, np.int32))
+    assert status == B.REFLEX_OK
+    assert np.all(np.isposinf(out))
