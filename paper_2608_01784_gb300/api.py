@@ -79,7 +79,8 @@ def update_state(state: dict, conf_new: torch.Tensor, num_blocks: torch.Tensor,
 
 
 def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
-                  flags: int = B.REFLEX_FLAG_RENORM_TOPK, count_rule: int = 0) -> int:
+                  flags: int = B.REFLEX_FLAG_RENORM_TOPK, count_rule: int = 0,
+                  k_max: int = 12) -> int:
     """Kernels one reflex_step call launches on the tcgen05 path, following the
     library's choices: the count kernel; the score kernel and the selection,
     or (bf16, renormalised weights, >= 128 experts, T E >= 2048 x 256,
@@ -89,7 +90,8 @@ def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
     the batched recheck; count + scan in one
     CTA (short batches whose block masks fit in shared memory) or count and
     scan, then the gather, which also places the pairs; the gate/up and down
-    GEMMs (and the shared expert's two); the combine.
+    GEMMs (and the shared expert's two, once the routed GEMMs run on CTA
+    pairs; the 1-SM launches carry its tiles); the combine.
     With a score count rule the selection derives the counts: no count
     kernel and no screen.  Memsets are not kernels."""
     n = 0 if count_rule else 1
@@ -100,7 +102,7 @@ def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
         (E <= 64 and T >= 8192) or (64 < E <= 256 and T >= 2048))
     n += 3 if (screen or batch_screen) else 2
     n += 1 if T <= 4096 and (T + 31) // 32 * E * 4 <= 160 * 1024 else 2
-    n += 1 + 2 + (2 if shared_inter else 0) + 1
+    n += 1 + 2 + (2 if shared_inter and T * k_max // 2 // E >= 128 else 0) + 1
     return n
 
 

@@ -93,6 +93,15 @@ struct KParams {
   int b3d;
   // scores mode, k_splits == 1: sum of squares of every A row (fp32), nullable
   float* norm_out;
+  // 1-SM kernel: a dense problem carried by the same launch (the shared
+  // expert): its sh_tiles tiles come first, sh_rows rows, n_tiles2 column
+  // tiles, reduction length K2, operands through map_a2 / map_b2
+  int sh_tiles;
+  int sh_rows;
+  int n_tiles2;
+  int K2;
+  __nv_bfloat16* out2;
+  int ldo2;
   // CTA pairs: whole 32-row output chunks leave by TMA store (map_out)
   int tma_out;
   // SwiGLU on CTA pairs: A rows gathered from the token rows (TcGemmArgs)
@@ -234,6 +243,7 @@ struct Tile {
   int e, n, row0, rows;
   int mtiles;  // m-tiles of the tile's group (readers of each weight tile)
   int ks;      // K slice (scores mode; 0 otherwise)
+  bool sh;     // tile of the dense problem that the launch carries along
 };
 
 // The group prefix arrays a tile lookup reads: copies in shared memory where
@@ -265,6 +275,7 @@ __device__ __forceinline__ TileIndex load_tile_index(const KParams& p, int32_t* 
   return ix;
 }
 
+template <bool SH>
 __device__ __forceinline__ int total_tiles(const KParams& p, const TileIndex& ix) {
   int mt;
   if (p.g.offsets == nullptr) {
@@ -274,12 +285,26 @@ __device__ __forceinline__ int total_tiles(const KParams& p, const TileIndex& ix
     if (mt < 0) mt = 0;
     if (mt > p.max_mtiles) mt = p.max_mtiles;
   }
-  return mt * p.n_tiles;
+  return mt * p.n_tiles + (SH ? p.sh_tiles : 0);
 }
 
 // Tile t -> (expert, n-tile, rows); false when the workspace is inconsistent.
+// SH: the launch carries a dense problem, whose tiles come first.
+template <bool SH>
 __device__ __forceinline__ bool decode_tile(const KParams& p, const TileIndex& ix, int t,
                                             Tile& o) {
+  o.sh = SH && t < p.sh_tiles;
+  if (o.sh) {
+    const int mt = (p.sh_rows + p.tile_rows - 1) / p.tile_rows;
+    o.ks = 0;
+    o.e = 0;
+    o.n = t / mt;
+    o.row0 = (t % mt) * p.tile_rows;
+    o.rows = min(p.tile_rows, p.sh_rows - o.row0);
+    o.mtiles = mt;
+    return true;
+  }
+  if (SH) t -= p.sh_tiles;
   if (p.g.offsets == nullptr) {
     const int mt = (p.g.dense_rows + p.tile_rows - 1) / p.tile_rows;
     const int per = mt * p.n_tiles;
@@ -310,11 +335,12 @@ __device__ __forceinline__ bool decode_tile(const KParams& p, const TileIndex& i
          o.row0 + o.rows <= p.g.cap_rows;
 }
 
-template <int BN, int MODE>
+template <int BN, int MODE, bool SH>
 __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThreads, 1)
     grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a,
                         const __grid_constant__ CUtensorMap map_b,
-                        const KParams p) {
+                        const __grid_constant__ CUtensorMap map_a2,
+                        const __grid_constant__ CUtensorMap map_b2, const KParams p) {
   using C = Cfg<BN>;
   constexpr int kStages = C::kStages;
   extern __shared__ uint8_t smem_raw[];
@@ -349,6 +375,10 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
     fence_mbar_init();
     prefetch_map(&map_a);
     prefetch_map(&map_b);
+    if (SH) {
+      prefetch_map(&map_a2);
+      prefetch_map(&map_b2);
+    }
   }
   if (warp == 1) tmem_alloc(smem_addr(tmem_slot), C::kTmemCols);
   tc_fence_before();
@@ -361,8 +391,9 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
   const TileIndex ix = load_tile_index(
       p, reinterpret_cast<int32_t*>(smem + kStages * C::kStageBytes + C::kBarBytes),
       C::kIndexInts);
-  const int ntiles = total_tiles(p, ix);
-  const int nk = p.K / BK / p.k_splits;  // k-blocks per tile
+  const int ntiles = total_tiles<SH>(p, ix);
+  const int nk_main = p.K / BK / p.k_splits, nk_sh = p.K2 / BK;  // k-blocks per tile
+  auto nk_of = [&](int t) { return SH && t < p.sh_tiles ? nk_sh : nk_main; };
 
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer ----------------
@@ -374,12 +405,15 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
     const uint64_t pol_once = l2_policy(kPolFirst);
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
       Tile tl;
-      if (!decode_tile(p, ix, t, tl)) {
+      if (!decode_tile<SH>(p, ix, t, tl)) {
         set_err(p.err, kErrIndex);
         *abort_flag = 1;
         break;
       }
       const bool once = grouped && tl.mtiles == 1;  // one reader per weight tile
+      const int nk = nk_of(t);
+      const CUtensorMap* ma = SH && tl.sh ? &map_a2 : &map_a;
+      const CUtensorMap* mb = SH && tl.sh ? &map_b2 : &map_b;
       for (int kb = 0; kb < nk; ++kb) {
         if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, kWaitNs)) {
           ok = false;
@@ -388,17 +422,17 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
         const uint32_t fb = smem_addr(&full[stage]);
         mbar_expect_tx(fb, C::kStageBytes);
         const int k0 = (tl.ks * nk + kb) * BK;
-        tma_load_2d(smem_addr(sa + stage * C::kABytes), &map_a, k0, tl.row0, fb);
+        tma_load_2d(smem_addr(sa + stage * C::kABytes), ma, k0, tl.row0, fb);
         const uint32_t b_dst = smem_addr(sb + stage * C::kBBytes);
         const int wr = tl.e * p.b_rows_per_group + tl.n * (MODE == kModeSwiGLU ? BN / 2 : BN);
         auto load_b = [&](uint32_t dst, int row) {
-          if (once) tma_load_2d_hint(dst, &map_b, k0, row, fb, pol_once);
-          else tma_load_2d(dst, &map_b, k0, row, fb);
+          if (once) tma_load_2d_hint(dst, mb, k0, row, fb, pol_once);
+          else tma_load_2d(dst, mb, k0, row, fb);
         };
         if (MODE == kModeSwiGLU && p.b3d) {
           // gate rows then up rows of the tile, one copy
-          if (once) tma_load_3d_hint(b_dst, &map_b, k0, tl.n * (BN / 2), 2 * tl.e, fb, pol_once);
-          else tma_load_3d(b_dst, &map_b, k0, tl.n * (BN / 2), 2 * tl.e, fb);
+          if (once) tma_load_3d_hint(b_dst, mb, k0, tl.n * (BN / 2), 2 * tl.e, fb, pol_once);
+          else tma_load_3d(b_dst, mb, k0, tl.n * (BN / 2), 2 * tl.e, fb);
         } else {
           load_b(b_dst, wr);
           if (MODE == kModeSwiGLU) load_b(b_dst + (BN / 2) * BK * 2, wr + p.b_up_offset);
@@ -437,6 +471,7 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
       }
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ab * BN);
+      const int nk = nk_of(t);
       for (int kb = 0; kb < nk; ++kb) {
         if (!mbar_wait(&full[stage], phase, abort_flag, kWaitNs)) {
           ok = false;
@@ -482,9 +517,9 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
       bool ok = true;
       for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
         Tile tl;
-        const bool tile_ok = decode_tile(p, ix, t, tl);
+        const bool tile_ok = decode_tile<SH>(p, ix, t, tl);
         float ss = 0.f;
-        for (int kb = 0; kb < nk; ++kb) {
+        for (int kb = 0; kb < nk_main; ++kb) {
           // every lane observes the stage's completion before reading it
           const bool w = __all_sync(0xffffffffu,
                                     mbar_wait(&full[stage], phase, abort_flag, kWaitNs));
@@ -529,7 +564,7 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
     int lt = 0;
     for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++lt) {
       Tile tl;
-      const bool tile_ok = decode_tile(p, ix, t, tl);
+      const bool tile_ok = decode_tile<SH>(p, ix, t, tl);
       const int ab = lt & 1;
       const uint32_t acc_phase = (lt >> 1) & 1;
       int ok = 1;
@@ -546,8 +581,9 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
       const uint32_t tbase = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
                              static_cast<uint32_t>(ab * BN);
       const bool store = tile_ok && row < tl.rows;
-      __nv_bfloat16* orow =
-          p.out + static_cast<int64_t>(tl.row0 + (store ? row : 0)) * p.ldo;
+      __nv_bfloat16* orow = (SH && tl.sh ? p.out2 : p.out) +
+                            static_cast<int64_t>(tl.row0 + (store ? row : 0)) *
+                                (SH && tl.sh ? p.ldo2 : p.ldo);
       if (MODE == kModeScores) {
         float* srow = p.out_f32 + tl.ks * p.split_stride +
                       static_cast<int64_t>(tl.row0 + (store ? row : 0)) * p.ldo;
@@ -635,10 +671,21 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
   if (p.defer_wait) grid_dep_wait();
 }
 
-template <int BN, int MODE>
+// The tiles of a dense problem (nullptr: none) that a 1-SM launch carries
+// along: `cols` output columns per tile.
+void set_shared_problem(KParams& p, const TcGemmArgs* sh, int cols) {
+  p.sh_rows = sh != nullptr ? sh->g.dense_rows : 0;
+  p.n_tiles2 = sh != nullptr ? sh->n_total / cols : 0;
+  p.K2 = sh != nullptr ? sh->K : 0;
+  p.out2 = sh != nullptr ? static_cast<__nv_bfloat16*>(sh->out) : nullptr;
+  p.ldo2 = sh != nullptr ? sh->ldo : 0;
+  p.sh_tiles = (p.sh_rows + p.tile_rows - 1) / p.tile_rows * p.n_tiles2;
+}
+
+template <int BN, int MODE, bool SH>
 cudaError_t launch_impl(const TcGemmArgs& a, cudaStream_t stream) {
   using C = Cfg<BN>;
-  auto kernel = grouped_gemm_kernel<BN, MODE>;
+  auto kernel = grouped_gemm_kernel<BN, MODE, SH>;
   cudaError_t e = cudaFuncSetAttribute(
       kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes);
   if (e != cudaSuccess) return e;
@@ -666,11 +713,13 @@ cudaError_t launch_impl(const TcGemmArgs& a, cudaStream_t stream) {
   p.gather_perm = nullptr;
   p.gather_kmax = 1;
   p.gather_tokens = 0;
-  const int64_t max_tiles = static_cast<int64_t>(p.n_tiles) * p.max_mtiles;
+  set_shared_problem(p, SH ? a.shared : nullptr, MODE == kModeSwiGLU ? BN / 2 : BN);
+  const int64_t max_tiles = static_cast<int64_t>(p.n_tiles) * p.max_mtiles + p.sh_tiles;
   if (max_tiles == 0) return cudaSuccess;
   const int grid = static_cast<int>(max_tiles < a.num_sms ? max_tiles : a.num_sms);
+  const TcGemmArgs& sh = SH ? *a.shared : a;
   return launch_pdl(kernel, dim3(grid), dim3(kThreads), C::kSmemBytes, stream, *a.map_a,
-                    *a.map_b, p);
+                    *a.map_b, *sh.map_a, *sh.map_b, p);
 }
 
 // ===========================================================================
@@ -902,7 +951,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
       load_tile_index(p, reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(bars) + 256),
                       C::kIndexInts);
   // tiles are 256 rows (both CTAs) x 256 columns; mt_prefix counts 256-row tiles
-  const int ntiles = total_tiles(p, ix);
+  const int ntiles = total_tiles<false>(p, ix);
   const int nk = p.K / (BK * C::KS);  // stages per tile
 
   // SwiGLU with gathered A rows: the whole producer warp issues the A
@@ -917,7 +966,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
     bool ok = true;
     for (int t = pair; t < ntiles && ok; t += npairs) {
       Tile tl;
-      if (!decode_tile(p, ix, t, tl)) {  // the same outcome in every lane
+      if (!decode_tile<false>(p, ix, t, tl)) {  // the same outcome in every lane
         if (lane == 0) {
           set_err(p.err, kErrIndex);
           *abort_flag = 1;
@@ -1088,7 +1137,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
     int lt = 0;
     for (int t = pair; t < ntiles; t += npairs, ++lt) {
       Tile tl;
-      const bool tile_ok = decode_tile(p, ix, t, tl);
+      const bool tile_ok = decode_tile<false>(p, ix, t, tl);
       const int ab = lt & 1;
       const uint32_t acc_phase = (lt >> 1) & 1;
       int ok = 1;
@@ -1206,6 +1255,7 @@ cudaError_t launch_pair_impl(const TcGemmArgs& a, cudaStream_t stream) {
   p.out = static_cast<__nv_bfloat16*>(a.out);
   p.ldo = a.ldo;
   p.err = a.err;
+  set_shared_problem(p, nullptr, C::BN);
   p.k_splits = 1;
   p.out_f32 = nullptr;
   p.split_stride = 0;
@@ -1245,20 +1295,26 @@ cudaError_t launch_pair_impl(const TcGemmArgs& a, cudaStream_t stream) {
 
 }  // namespace
 
+template <int MODE>
+cudaError_t launch_any(const TcGemmArgs& a, int bn, cudaStream_t stream) {
+  if (a.shared != nullptr)
+    return bn == 128 ? launch_impl<128, MODE, true>(a, stream)
+                     : launch_impl<256, MODE, true>(a, stream);
+  return bn == 128 ? launch_impl<128, MODE, false>(a, stream)
+                   : launch_impl<256, MODE, false>(a, stream);
+}
 cudaError_t launch_swiglu_tc(const TcGemmArgs& a, int bn, cudaStream_t stream) {
-  if (bn == 128) return launch_impl<128, kModeSwiGLU>(a, stream);
-  return launch_impl<256, kModeSwiGLU>(a, stream);
+  return launch_any<kModeSwiGLU>(a, bn, stream);
 }
 cudaError_t launch_down_tc(const TcGemmArgs& a, int bn, cudaStream_t stream) {
-  if (bn == 128) return launch_impl<128, kModeDown>(a, stream);
-  return launch_impl<256, kModeDown>(a, stream);
+  return launch_any<kModeDown>(a, bn, stream);
 }
 template <int BN>
 cudaError_t launch_scores_impl(const TcGemmArgs& a, int k_splits, float* out,
                                int64_t split_stride, int n_valid, bool defer_wait,
                                float* row_norms, cudaStream_t stream) {
   using C = Cfg<BN>;
-  auto kernel = grouped_gemm_kernel<BN, kModeScores>;
+  auto kernel = grouped_gemm_kernel<BN, kModeScores, false>;
   if (a.g.offsets != nullptr || k_splits < 1 || (a.K / BK) % k_splits != 0 ||
       a.K % BK != 0 || n_valid < 1 || (row_norms != nullptr && k_splits != 1))
     return cudaErrorInvalidValue;
@@ -1288,7 +1344,7 @@ cudaError_t launch_scores_impl(const TcGemmArgs& a, int k_splits, float* out,
   if (max_tiles == 0) return cudaSuccess;
   const int grid = static_cast<int>(max_tiles < a.num_sms ? max_tiles : a.num_sms);
   return launch_pdl(kernel, dim3(grid), dim3(kThreadsScores), C::kSmemBytes, stream,
-                    *a.map_a, *a.map_b, p);
+                    *a.map_a, *a.map_b, *a.map_a, *a.map_b, p);
 }
 
 // SwiGLU loads gate and up halves as two boxes of bn/2 rows; down loads one

@@ -207,6 +207,10 @@ struct TcGemmArgs {
   // swizzle; whole 32-row output chunks are written by TMA stores through it
   // (nullptr: per-lane stores)
   const CUtensorMap* map_out = nullptr;
+  // 1-SM kernels, grouped rows: a dense problem (the shared expert) whose
+  // tiles the same launch computes; map_b of the kind of this one, n_total a
+  // multiple of the tile's columns
+  const TcGemmArgs* shared = nullptr;
 };
 // SwiGLU: out = silu(A Wg^T) * (A Wu^T).  Down: out = A Wd^T.  bn = tile
 // width (128 or 256, from tc_pick_bn); the B tensor map's box must have

@@ -572,18 +572,27 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
       // 256 pair tile moves a quarter of the operand bytes per output that a
       // 128 x 128 tile of the 1-SM kernel moves from L2 (LLaDA2.0-mini layer
       // 0.750 -> 0.736 ms; at 1024 tokens the 1-SM tiles stay 6 us faster)
-      const bool pair_shared =
-          shared_inter > 0 && T >= 2048 && shared_inter % 128 == 0 && d % 256 == 0;
+      // With 1-SM routed GEMMs the shared expert's tiles ride in the routed
+      // launches: alone they take a K-long latency on a few SMs, there they
+      // hide behind the weight stream (LLaDA2.0-mini shape: 16 tokens 162 ->
+      // 143 us, 256 308 -> 289, 1024 359 -> 337, 4096 486 -> 470).  CTA-pair
+      // launches carried them without a gain (8192 tokens 0.547 / 0.548 ms)
+      const bool carry_shared = shared_inter > 0 && !pair_routed &&
+                                shared_inter % rx::tc_n_granule(true, bn_up) == 0 &&
+                                d % rx::tc_n_granule(false, bn_dn) == 0;
+      const bool pair_shared = shared_inter > 0 && !carry_shared && T >= 2048 &&
+                               shared_inter % 128 == 0 && d % 256 == 0;
+      const int bn_s1 = carry_shared ? bn_up : bn_sup, bn_s2 = carry_shared ? bn_dn : bn_sdn;
       CUtensorMap sa1, sb1, sa2, sb2;
       if (shared_inter &&
           (!make_map(&sa1, hidden, T, d, rx::kTileM) ||
            !(pair_shared
                  ? make_map(&sb1, shared_gate_up, 2 * static_cast<int64_t>(shared_inter), d, 128)
                  : make_map_gate_up(&sb1, shared_gate_up, 1, shared_inter, d,
-                                    rx::tc_b_box_rows(true, bn_sup))) ||
+                                    rx::tc_b_box_rows(true, bn_s1))) ||
            !make_map(&sa2, ash, T, shared_inter, rx::kTileM) ||
            !make_map(&sb2, shared_down, d, shared_inter,
-                     pair_shared ? 128 : rx::tc_b_box_rows(false, bn_sdn))))
+                     pair_shared ? 128 : rx::tc_b_box_rows(false, bn_s2))))
         return REFLEX_ECUDA;
       rx::TcGemmArgs h1{&sa1, &sb1, d, shared_inter, 2 * shared_inter, shared_inter,
                         dense, ash, shared_inter, err, sms, !pair_shared};
@@ -595,12 +604,17 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
         h1.map_out = &so1;
         h2.map_out = &so2;
       }
+      if (carry_shared) {
+        g1.shared = &h1;
+        g2.shared = &h2;
+      }
+      const bool own_shared = shared_inter > 0 && !carry_shared;
       if (up) {
         if (pair_routed)
           RX_CUDA(rx::launch_swiglu_tc_pair(g1, s));
         else
           RX_CUDA(rx::launch_swiglu_tc(g1, bn_up, s));
-        if (shared_inter) {
+        if (own_shared) {
           if (pair_shared)
             RX_CUDA(rx::launch_swiglu_tc_pair(h1, s));
           else
@@ -612,7 +626,7 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
           RX_CUDA(rx::launch_down_tc_pair(g2, s));
         else
           RX_CUDA(rx::launch_down_tc(g2, bn_dn, s));
-        if (shared_inter) {
+        if (own_shared) {
           if (pair_shared)
             RX_CUDA(rx::launch_down_tc_pair(h2, s));
           else
