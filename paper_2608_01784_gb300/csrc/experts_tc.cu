@@ -102,6 +102,9 @@ struct KParams {
   int K2;
   __nv_bfloat16* out2;
   int ldo2;
+  // 1: the first ring stages' weights are requested before the dependency
+  // wait (early_tile)
+  int early_b;
   // CTA pairs: whole 32-row output chunks leave by TMA store (map_out)
   int tma_out;
   // SwiGLU on CTA pairs: A rows gathered from the token rows (TcGemmArgs)
@@ -114,6 +117,11 @@ struct KParams {
 __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar),
                "r"(bytes)
+               : "memory");
+}
+// Announces bytes on a phase whose arrival comes later (another expect_tx).
+__device__ __forceinline__ void mbar_expect_tx_only(uint32_t bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cta.shared::cta.b64 [%0], %1;" ::"r"(bar), "r"(bytes)
                : "memory");
 }
 __device__ __forceinline__ void mbar_arrive1(uint32_t bar) {
@@ -335,6 +343,47 @@ __device__ __forceinline__ bool decode_tile(const KParams& p, const TileIndex& i
          o.row0 + o.rows <= p.g.cap_rows;
 }
 
+// Expert, n-tile and m-tile count of tile t, read before the kernel's
+// dependency wait, by a whole warp (a 32-ary search: one or two rounds of L2
+// loads).  The host asks for it (early_b) only where the kernel in front of
+// this one in the stream waited for the dispatch itself before it let this
+// one launch, so the prefix is complete; the operand that the kernel in front
+// writes (A) is not touched.  False: no such tile.
+template <bool SH>
+__device__ __forceinline__ bool early_tile(const KParams& p, int t, Tile& o) {
+  o.sh = SH && t < p.sh_tiles;
+  if (o.sh) {
+    const int mt = (p.sh_rows + p.tile_rows - 1) / p.tile_rows;
+    o.e = 0;
+    o.n = t / mt;
+    o.mtiles = mt;
+    return true;
+  }
+  if (SH) t -= p.sh_tiles;
+  if (p.g.offsets == nullptr) {
+    const int mt = (p.g.dense_rows + p.tile_rows - 1) / p.tile_rows;
+    o.e = 0;
+    o.n = t / mt;
+    o.mtiles = mt;
+    return o.n < p.n_tiles;
+  }
+  const int lane = threadIdx.x & 31;
+  int lo = 0, n = p.g.E;
+  while (n > 1) {
+    const int step = (n + 31) / 32;
+    const bool below = lane * step < n && p.n_tiles * __ldcg(p.mt_prefix + lo + lane * step) <= t;
+    const int hit = 31 - __clz(__ballot_sync(0xffffffffu, below) | 1u);
+    lo += hit * step;
+    n = min(step, n - hit * step);
+  }
+  const int first = __ldcg(p.mt_prefix + lo), mt = __ldcg(p.mt_prefix + lo + 1) - first;
+  if (mt <= 0 || t < p.n_tiles * first) return false;
+  o.e = lo;
+  o.n = (t - p.n_tiles * first) / mt;
+  o.mtiles = mt;
+  return o.n < p.n_tiles;
+}
+
 template <int BN, int MODE, bool SH>
 __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThreads, 1)
     grouped_gemm_kernel(const __grid_constant__ CUtensorMap map_a,
@@ -380,6 +429,49 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
       prefetch_map(&map_b2);
     }
   }
+  const int nk_main = p.K / BK / p.k_splits, nk_sh = p.K2 / BK;  // k-blocks per tile
+  auto nk_of = [&](int t) { return SH && t < p.sh_tiles ? nk_sh : nk_main; };
+  const uint64_t pol_once = l2_policy(kPolFirst);
+  // the weight tile of k-block kb of tile tl into stage s
+  auto load_weights = [&](const Tile& tl, bool once, int kb, int s, int nk) {
+    const uint32_t fb = smem_addr(&full[s]);
+    const uint32_t b_dst = smem_addr(sb + s * C::kBBytes);
+    const CUtensorMap* mb = SH && tl.sh ? &map_b2 : &map_b;
+    const int k0 = (tl.ks * nk + kb) * BK;
+    const int wr = tl.e * p.b_rows_per_group + tl.n * (MODE == kModeSwiGLU ? BN / 2 : BN);
+    auto load_b = [&](uint32_t dst, int row) {
+      if (once) tma_load_2d_hint(dst, mb, k0, row, fb, pol_once);
+      else tma_load_2d(dst, mb, k0, row, fb);
+    };
+    if (MODE == kModeSwiGLU && p.b3d) {
+      // gate rows then up rows of the tile, one copy
+      if (once) tma_load_3d_hint(b_dst, mb, k0, tl.n * (BN / 2), 2 * tl.e, fb, pol_once);
+      else tma_load_3d(b_dst, mb, k0, tl.n * (BN / 2), 2 * tl.e, fb);
+    } else {
+      load_b(b_dst, wr);
+      if (MODE == kModeSwiGLU) load_b(b_dst + (BN / 2) * BK * 2, wr + p.b_up_offset);
+    }
+  };
+  // The ring's first weights while the kernel in front still runs: the
+  // stream starts a ring earlier (32 tokens of the LLaDA-MoE shape 162 -> 158
+  // us, 16 of the LLaDA2.0-mini shape 143 -> 137, 1024 337 -> 330)
+  int early = 0;  // stages whose weights are on their way (warp 0)
+  if (MODE != kModeScores && p.early_b && warp == 0) {
+    __syncwarp();
+    Tile tl;
+    if (early_tile<SH>(p, blockIdx.x, tl)) {
+      tl.ks = 0;
+      const int nk = nk_of(blockIdx.x);
+      early = nk < kStages ? nk : kStages;
+      const bool once = p.g.offsets != nullptr && tl.mtiles == 1;
+      if (lane == 0) {
+        for (int s = 0; s < early; ++s) {
+          mbar_expect_tx_only(smem_addr(&full[s]), C::kBBytes);
+          load_weights(tl, once, s, s, nk);
+        }
+      }
+    }
+  }
   if (warp == 1) tmem_alloc(smem_addr(tmem_slot), C::kTmemCols);
   tc_fence_before();
   __syncthreads();
@@ -392,8 +484,6 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
       p, reinterpret_cast<int32_t*>(smem + kStages * C::kStageBytes + C::kBarBytes),
       C::kIndexInts);
   const int ntiles = total_tiles<SH>(p, ix);
-  const int nk_main = p.K / BK / p.k_splits, nk_sh = p.K2 / BK;  // k-blocks per tile
-  auto nk_of = [&](int t) { return SH && t < p.sh_tiles ? nk_sh : nk_main; };
 
   if (warp == 0 && lane == 0) {
     // ---------------- TMA producer ----------------
@@ -402,7 +492,6 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
     uint32_t issued_mask = 0, issued_phase = 0;
     bool ok = true;
     const bool grouped = p.g.offsets != nullptr;
-    const uint64_t pol_once = l2_policy(kPolFirst);
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
       Tile tl;
       if (!decode_tile<SH>(p, ix, t, tl)) {
@@ -413,30 +502,18 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
       const bool once = grouped && tl.mtiles == 1;  // one reader per weight tile
       const int nk = nk_of(t);
       const CUtensorMap* ma = SH && tl.sh ? &map_a2 : &map_a;
-      const CUtensorMap* mb = SH && tl.sh ? &map_b2 : &map_b;
       for (int kb = 0; kb < nk; ++kb) {
         if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, kWaitNs)) {
           ok = false;
           break;
         }
         const uint32_t fb = smem_addr(&full[stage]);
-        mbar_expect_tx(fb, C::kStageBytes);
         const int k0 = (tl.ks * nk + kb) * BK;
+        const bool ahead = early > 0;  // the weights are already on their way
+        mbar_expect_tx(fb, ahead ? C::kABytes : C::kStageBytes);
         tma_load_2d(smem_addr(sa + stage * C::kABytes), ma, k0, tl.row0, fb);
-        const uint32_t b_dst = smem_addr(sb + stage * C::kBBytes);
-        const int wr = tl.e * p.b_rows_per_group + tl.n * (MODE == kModeSwiGLU ? BN / 2 : BN);
-        auto load_b = [&](uint32_t dst, int row) {
-          if (once) tma_load_2d_hint(dst, mb, k0, row, fb, pol_once);
-          else tma_load_2d(dst, mb, k0, row, fb);
-        };
-        if (MODE == kModeSwiGLU && p.b3d) {
-          // gate rows then up rows of the tile, one copy
-          if (once) tma_load_3d_hint(b_dst, mb, k0, tl.n * (BN / 2), 2 * tl.e, fb, pol_once);
-          else tma_load_3d(b_dst, mb, k0, tl.n * (BN / 2), 2 * tl.e, fb);
-        } else {
-          load_b(b_dst, wr);
-          if (MODE == kModeSwiGLU) load_b(b_dst + (BN / 2) * BK * 2, wr + p.b_up_offset);
-        }
+        if (ahead) --early;
+        else load_weights(tl, once, kb, stage, nk);
         issued_mask |= 1u << stage;
         issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
         if (++stage == kStages) {
@@ -448,6 +525,14 @@ __global__ void __launch_bounds__(MODE == kModeScores ? kThreadsScores : kThread
     if (!ok) {
       set_err(p.err, kErrTimeout);
       *abort_flag = 1;
+    }
+    // weights requested early for stages that never got their rows (no tile,
+    // or an error): the phase completes with the arrival that is missing
+    const int unused = early;
+    for (int s = 0; s < unused; ++s) {
+      const int st = (stage + s) % kStages;
+      mbar_arrive1(smem_addr(&full[st]));
+      mbar_wait(&full[st], 0, nullptr, kDrainNs);
     }
     if (*abort_flag) {
       // every issued load must land before the CTA may exit
@@ -707,6 +792,7 @@ cudaError_t launch_impl(const TcGemmArgs& a, cudaStream_t stream) {
   p.split_stride = 0;
   p.n_valid = 0;
   p.defer_wait = 0;
+  p.early_b = a.early_b ? 1 : 0;
   p.b3d = MODE == kModeSwiGLU && a.b_gate_up_3d ? 1 : 0;
   p.norm_out = nullptr;
   p.tma_out = 0;
@@ -768,6 +854,11 @@ __device__ __forceinline__ uint32_t map_to_rank(uint32_t addr, uint32_t rank) {
 // release needed (the bytes themselves arrive by TMA complete_tx).
 __device__ __forceinline__ void mbar_expect_tx_cluster(uint32_t cl_bar, uint32_t bytes) {
   asm volatile("mbarrier.arrive.expect_tx.relaxed.cluster.shared::cluster.b64 _, [%0], %1;" ::"r"(cl_bar),
+               "r"(bytes)
+               : "memory");
+}
+__device__ __forceinline__ void mbar_expect_tx_only_cluster(uint32_t cl_bar, uint32_t bytes) {
+  asm volatile("mbarrier.expect_tx.relaxed.cluster.shared::cluster.b64 [%0], %1;" ::"r"(cl_bar),
                "r"(bytes)
                : "memory");
 }
@@ -940,6 +1031,32 @@ __global__ void __launch_bounds__(kThreads2, 1)
     if (p.tma_out) prefetch_map(&map_out);
   }
   cluster_sync_all();  // barriers of both CTAs initialised; the peer is running
+  const int nk = p.K / (BK * C::KS);  // stages per tile
+  // first weight row of this CTA's half of tile (e, n)
+  auto weight_row = [&](const Tile& tl) {
+    return MODE == kModeSwiGLU
+               ? tl.e * p.b_rows_per_group + (rank ? p.b_up_offset : 0) + tl.n * (BN / 2)
+               : tl.e * p.b_rows_per_group + tl.n * BN + static_cast<int>(rank) * (BN / 2);
+  };
+  // the ring's first weights while the kernel in front still runs, as in the
+  // 1-SM kernel; both CTAs' bytes count on the leader's barriers
+  int early = 0;  // stages whose weights are on their way (warp 0)
+  if (p.early_b && p.gather_perm == nullptr && warp == 0) {
+    Tile tl;
+    if (early_tile<false>(p, pair, tl)) {
+      early = nk < kStages ? nk : kStages;
+      if (lane == 0) {
+        for (int s = 0; s < early; ++s) {
+          const uint32_t fb = map_to_rank(smem_addr(&full[s]), 0);
+          if (leader) mbar_expect_tx_only(smem_addr(&full[s]), C::kBBytes);
+          else mbar_expect_tx_only_cluster(fb, C::kBBytes);
+          for (int u = 0; u < C::KS; ++u)
+            tma_load_2d_pair(smem_addr(sb + s * C::kBBytes + u * C::kSubBytes), &map_b,
+                             (s * C::KS + u) * BK, weight_row(tl), fb);
+        }
+      }
+    }
+  }
   if (warp == 1) tmem_alloc_pair(smem_addr(tmem_slot), C::kTmemCols);
   tc_fence_before();
   __syncthreads();
@@ -952,7 +1069,6 @@ __global__ void __launch_bounds__(kThreads2, 1)
                       C::kIndexInts);
   // tiles are 256 rows (both CTAs) x 256 columns; mt_prefix counts 256-row tiles
   const int ntiles = total_tiles<false>(p, ix);
-  const int nk = p.K / (BK * C::KS);  // stages per tile
 
   // SwiGLU with gathered A rows: the whole producer warp issues the A
   // copies, one four-row gather per lane and 64-k block (lane l: rows 4 l ..
@@ -996,16 +1112,15 @@ __global__ void __launch_bounds__(kThreads2, 1)
           break;
         }
         const uint32_t fb = map_to_rank(smem_addr(&full[stage]), 0);
-        int brow;
-        if (MODE == kModeSwiGLU)
-          brow = tl.e * p.b_rows_per_group + (rank ? p.b_up_offset : 0) + tl.n * (BN / 2);
-        else
-          brow = tl.e * p.b_rows_per_group + tl.n * BN + static_cast<int>(rank) * (BN / 2);
+        const int brow = weight_row(tl);
+        const bool ahead = early > 0;  // the weights are already on their way
+        if (ahead) --early;
         if (lane == 0) {
+          const uint32_t bytes = ahead ? C::kABytes : C::kStageBytes;
           if (leader)
-            mbar_expect_tx(smem_addr(&full[stage]), C::kStageBytes);
+            mbar_expect_tx(smem_addr(&full[stage]), bytes);
           else
-            mbar_expect_tx_cluster(fb, C::kStageBytes);
+            mbar_expect_tx_cluster(fb, bytes);
           // consecutive k blocks of the same rows back to back
 #pragma unroll
           for (int u = 0; u < C::KS; ++u) {
@@ -1013,8 +1128,9 @@ __global__ void __launch_bounds__(kThreads2, 1)
             if (!gather)
               tma_load_2d_pair(smem_addr(sa + stage * C::kABytes + u * C::kSubBytes), &map_a,
                                k0, tl.row0 + static_cast<int>(rank) * BM, fb);
-            tma_load_2d_pair(smem_addr(sb + stage * C::kBBytes + u * C::kSubBytes), &map_b, k0,
-                             brow, fb);
+            if (!ahead)
+              tma_load_2d_pair(smem_addr(sb + stage * C::kBBytes + u * C::kSubBytes), &map_b, k0,
+                               brow, fb);
           }
         }
         if (gather) {
@@ -1037,6 +1153,17 @@ __global__ void __launch_bounds__(kThreads2, 1)
       if (!ok) {
         set_err(p.err, kErrTimeout);
         *abort_flag = 1;
+      }
+      // early weights of stages that never got their rows: both CTAs arrive,
+      // and the leader sees the bytes of both land
+      for (int s = 0; s < early; ++s) {
+        const int st = (stage + s) % kStages;
+        if (leader) {
+          mbar_arrive1(smem_addr(&full[st]));
+          mbar_wait(&full[st], 0, nullptr, kDrainNs);
+        } else {
+          mbar_arrive_cluster_relaxed(map_to_rank(smem_addr(&full[st]), 0));
+        }
       }
       if (*abort_flag && leader) {
         for (int s = 0; s < kStages; ++s)
@@ -1261,6 +1388,7 @@ cudaError_t launch_pair_impl(const TcGemmArgs& a, cudaStream_t stream) {
   p.split_stride = 0;
   p.n_valid = 0;
   p.defer_wait = 0;
+  p.early_b = a.early_b ? 1 : 0;
   p.b3d = 0;
   p.norm_out = nullptr;
   p.tma_out = a.map_out != nullptr ? 1 : 0;

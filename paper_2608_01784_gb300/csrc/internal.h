@@ -211,6 +211,10 @@ struct TcGemmArgs {
   // tiles the same launch computes; map_b of the kind of this one, n_total a
   // multiple of the tile's columns
   const TcGemmArgs* shared = nullptr;
+  // the kernel in front of this one in the stream waited for the dispatch
+  // (the tile prefix) before it let this launch start: the first weights may
+  // be requested before this kernel's own wait
+  bool early_b = false;
 };
 // SwiGLU: out = silu(A Wg^T) * (A Wu^T).  Down: out = A Wd^T.  bn = tile
 // width (128 or 256, from tc_pick_bn); the B tensor map's box must have

@@ -609,6 +609,11 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
         g2.shared = &h2;
       }
       const bool own_shared = shared_inter > 0 && !carry_shared;
+      // weights ahead of the dependency wait only behind a kernel of this call
+      // that itself waited for the dispatch: the gather (which waits for the
+      // scan), then the GEMMs in turn
+      g1.early_b = (stages & REFLEX_STAGE_DISPATCH) != 0;
+      h1.early_b = g2.early_b = h2.early_b = up;
       if (up) {
         if (pair_routed)
           RX_CUDA(rx::launch_swiglu_tc_pair(g1, s));
