@@ -106,7 +106,7 @@ cudaError_t launch_router_screen_batch(const CUtensorMap* map_h, const CUtensorM
                                        float* z, const float* hss, const float* nw,
                                        const int32_t* k, int T, int E, int d, int k_max,
                                        int32_t* ids, float* alpha, uint32_t* err,
-                                       cudaStream_t stream);
+                                       int num_sms, cudaStream_t stream);
 // The counts from the router scores (count rules 1 = Top-p, 2 = expert
 // threshold, threshold thr, clip [k_lo, min(k_hi, E)]) into k_out (and added
 // to k_sum, nullable, which the caller cleared), then ids / alpha [T, k_max]

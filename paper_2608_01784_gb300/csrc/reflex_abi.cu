@@ -21,11 +21,16 @@ using rx::WsHeader;
 constexpr size_t kAlign = 256;
 // gate/up weight bytes handed to the L2 while the router scores run
 constexpr uint64_t kRouterL2Prefetch = 64ull << 20;
-// tokens from which layers with up to 64 experts screen their router scores
-constexpr int32_t kBatchScreenMinTokens = 8192;      // up to 64 experts
-// 65 to 256 experts: from 2048 tokens, where the per-token recheck starts
-// (LLaDA2.0-mini shape: 2048 tokens 0.413 -> 0.394 ms, 4096 0.495 -> 0.478)
-constexpr int32_t kBatchScreenMinTokensWide = 2048;
+// Scores T E from which layers with up to 256 experts screen their router
+// scores in batches: the dense chains cost T E, the screen's three kernels
+// about 40 us at least, and with few experts most of a token's work is the
+// screen itself.  Layer times dense / screened: 256 experts, 1024 tokens 329
+// / 326 us; 160, 1300: 244.5 / 243.7; 96, 2048: 231 / 228; 64, 3270: 377 /
+// 376, 6000: 540 / 526; 32, 8192: 408 / 412; 16, 8192: 382 / 402, 16000: 707
+// / 713; 8, 16000: 663 / 687.
+int64_t batch_screen_min_scores(int32_t E) {
+  return E <= 32 ? 16384 * 32 : E <= 64 ? 4608 * 64 : 768 * 256;
+}
 constexpr int32_t kBatchScreenMaxExperts = 256;
 size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
 
@@ -114,9 +119,10 @@ PFN_cuTensorMapEncodeTiled_v12000 encode_fn() {
 }
 
 // 2-D bf16 map over a row-major [rows, cols] matrix; box = 64 columns (128
-// bytes, one swizzle row) x box_rows rows, 128-byte swizzle, zero fill.
+// bytes, one swizzle row) x box_rows rows, 128-byte swizzle unless another is
+// given, zero fill.
 bool make_map(CUtensorMap* m, const void* base, int64_t rows, int64_t cols,
-              int box_rows) {
+              int box_rows, CUtensorMapSwizzle swizzle = CU_TENSOR_MAP_SWIZZLE_128B) {
   auto fn = encode_fn();
   if (fn == nullptr) return false;
   if ((reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
@@ -126,7 +132,7 @@ bool make_map(CUtensorMap* m, const void* base, int64_t rows, int64_t cols,
   cuuint32_t estr[2] = {1, 1};
   CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base),
                   dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  swizzle, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
                   CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS;
 }
@@ -445,13 +451,15 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
   const bool batch_screen = dtype == REFLEX_DTYPE_BF16 && (flags & REFLEX_FLAG_RENORM_TOPK) &&
                             !(flags & REFLEX_FLAG_EXACT_SCORES) && !rule &&
                             E <= kBatchScreenMaxExperts && d % 64 == 0 &&
-                            T >= (E <= 64 ? kBatchScreenMinTokens : kBatchScreenMinTokensWide);
+                            static_cast<int64_t>(T) * E >= batch_screen_min_scores(E);
   if ((stages & REFLEX_STAGE_ROUTE) && batch_screen) {
     CUtensorMap mh, mw, mhb, mwb;
     const int sbn = E <= 64 ? 64 : 128;  // score tile width
     if (!make_map(&mh, hidden, T, d, rx::kTileM) || !make_map(&mw, w_router, E, d, sbn) ||
-        !make_map(&mhb, hidden, T, d, rx::screen_batch_token_rows(E)) ||
-        !make_map(&mwb, w_router, E, d, rx::screen_batch_expert_rows(E)))
+        !make_map(&mhb, hidden, T, d, rx::screen_batch_token_rows(E),
+                  CU_TENSOR_MAP_SWIZZLE_NONE) ||
+        !make_map(&mwb, w_router, E, d, rx::screen_batch_expert_rows(E),
+                  CU_TENSOR_MAP_SWIZZLE_NONE))
       return REFLEX_ECUDA;
     float* nw = reinterpret_cast<float*>(ws + L.wnorm);
     float* hss = reinterpret_cast<float*>(ws + L.tnorm);
@@ -463,7 +471,7 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
     RX_CUDA(rx::launch_scores_tc(sa, sbn, 1, z, static_cast<int64_t>(T) * E, E, true, s, hss));
     if (ac != nullptr) RX_CUDA(launch_alloc(*ac, T, s, true));
     RX_CUDA(rx::launch_router_screen_batch(&mhb, &mwb, z, hss, nw, k, T, E, d, k_max,
-                                           I32(L.ids), alpha, err, s));
+                                           I32(L.ids), alpha, err, sms, s));
   } else if ((stages & REFLEX_STAGE_ROUTE) && screen) {
     const int bn = rx::screen_bn(E), ks = rx::screen_splits(T, E, d);
     CUtensorMap mh, mw;

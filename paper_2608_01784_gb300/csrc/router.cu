@@ -1165,8 +1165,7 @@ __global__ void __launch_bounds__(kScreenWarps * 32)
 // to 64 experts; at 32 x 1024 tokens 1024 CTAs spread evenly over the SMs,
 // where 64-token CTAs, two per SM, left some SMs idle for half of the
 // kernel and 16-token CTAs stream the expert rows too often):
-//   1. screening (8 warps, the CTA's tokens in turn, up to four tokens'
-//      rounds interleaved):
+//   1. screening (a warp per token, up to four tokens' rounds interleaved):
 //      from the tensor-core estimates z~ and the row norms (the score GEMM's
 //      sums of squares, ||w_e|| from wnorm_kernel) the interval z~ -/+ del
 //      of every (token, expert), the k_t-th largest lower end L, and the
@@ -1174,60 +1173,73 @@ __global__ void __launch_bounds__(kScreenWarps * 32)
 //      the tokens lays the (token, expert) candidate pairs out in shared
 //      memory;
 //   2. chains: a producer warp streams 64-k chunks of the CTA's token rows
-//      and of the 32 NPL expert rows through a TMA ring (128-byte
-//      swizzle); each compute thread advances the canonical fma chain of two
-//      candidate pairs over the chunk, the pairs laid out so that a quarter
-//      warp's expert rows fall in distinct bank groups (more than 512 pairs:
-//      the rows are streamed again for the next 512);
+//      and of the 32 NPL expert rows through a TMA ring; each compute thread
+//      advances the canonical fma chains of two candidates of one token over
+//      the chunk, the lanes skewed by a 16-byte step each so that no two of a
+//      quarter warp meet in a bank (more duos than threads: the rows are
+//      streamed again for the next);
 //   3. selection (a warp per token): TopK over the candidates' exact
 //      scores by rank counting, with the keys and tie rule of select_kernel,
 //      the weights with its arithmetic (the same bits), and the exact scores
 //      into z.
-constexpr int kBatchCompute = 256;            // 8 compute warps
-constexpr int kBatchThreads = kBatchCompute + 32;  // + the producer warp
-constexpr int kBatchSlots = 2 * kBatchCompute;     // candidate pairs per pass
 constexpr uint64_t kBatchWaitNs = 2000000000ull;
 constexpr uint64_t kBatchDrainNs = 1000000000ull;
 // NPL groups of 32 experts: every lane of a screening warp holds NPL of a
-// token's experts, and every stage holds the 32 NPL expert rows.  Up to 64
-// experts (NPL 2): 32 tokens per CTA, three CTAs per SM, four tokens'
-// rounds interleaved per warp; up to 256 (NPL 8): 16 tokens per CTA, a
-// 2-stage ring, two CTAs per SM, one token at a time (LLaDA2.0-mini layer
-// 0.553 ms with 32 tokens and one CTA per SM, 0.558 with 16 and one, 0.546
-// with 16 and two).
+// token's experts, and every stage holds the 32 NPL expert rows.
+//   up to 64 experts (NPL 2): 32 tokens and 8 compute warps per CTA, three
+//   CTAs per SM, four tokens' rounds interleaved per warp;
+//   up to 256 (NPL 8): up to 64 tokens and 16 compute warps, one CTA per SM,
+//   a 4-stage ring.  Each CTA streams all 256 expert rows (1 MB at d = 2048),
+//   so the tokens per CTA set how often an SM takes them in: with 16 tokens
+//   the rows' way into the SMs (64 bytes per cycle) bounded the kernel
+//   (65536 tokens: 445 us with 16 tokens per CTA, 351 with 64; with the
+//   skewed duo chains and the sorted rounds below 241; 8192 tokens 67 -> 61
+//   -> 40; 32768 tokens x 64 experts, 32 tokens per CTA in each: 120 -> 85;
+//   40 or 56 tokens per CTA or four CTAs per SM there: no faster).
 template <int NPL>
 struct BatchCfg {
-  static constexpr int kT = NPL <= 2 ? 32 : 16;       // tokens per CTA
+  static constexpr int kT = NPL <= 2 ? 32 : 64;       // most tokens per CTA
+  static constexpr int kWarps = NPL <= 2 ? 8 : 16;    // compute warps
+  static constexpr int kCompute = 32 * kWarps;
+  static constexpr int kThreads = kCompute + 32;      // + the producer warp
   static constexpr int kE = 32 * NPL;                 // expert rows per stage
-  static constexpr int kStages = NPL <= 2 ? 4 : 2;
-  static constexpr int kMinCtas = NPL <= 2 ? 3 : 2;   // co-resident CTAs per SM
-  static constexpr int kGroup = NPL <= 2 ? 4 : 1;     // tokens whose rounds interleave
+  static constexpr int kStages = 4;
+  static constexpr int kMinCtas = NPL <= 2 ? 3 : 1;   // co-resident CTAs per SM
+  static constexpr int kGroup = NPL <= 2 ? 4 : 2;     // tokens whose rounds interleave
   static constexpr int kIdBits = NPL <= 2 ? 6 : 8;    // expert index bits of a key
+  // candidate pairs held at a time; a block with more runs its chains and
+  // selection in rounds of consecutive tokens
+  static constexpr int kCap = 2048;
   static constexpr uint32_t kTokBytes = kT * 128;
   static constexpr uint32_t kStageBytes = kTokBytes + kE * 128;
   static_assert(kT % 8 == 0 && kT <= 64, "whole swizzle atoms; the prefix's 64 lanes");
+  static_assert(kCap >= kE, "a round holds at least one token");
 };
 template <int NPL>
 struct BatchSmem {
-  static constexpr int kT = BatchCfg<NPL>::kT;
-  uint64_t full[BatchCfg<NPL>::kStages];
-  uint64_t empty[BatchCfg<NPL>::kStages];
-  uint32_t mask[kT][NPL];
-  int32_t cnt[kT];
-  int32_t kt[kT];
-  int32_t off[kT + 1];
-  float sel_z[8][32];
-  int32_t sel_e[8][32];
+  using C = BatchCfg<NPL>;
+  uint64_t full[C::kStages];
+  uint64_t empty[C::kStages];
+  uint32_t mask[C::kT][NPL];
+  int32_t cnt[C::kT];
+  int32_t kt[C::kT];
+  int32_t off[C::kT + 1];   // first candidate pair of each token, the total
+  int32_t doff[C::kT + 1];  // first duo (two pairs of one token)
+  float sel_z[C::kWarps][32];
+  int32_t sel_e[C::kWarps][32];
   volatile int abort;
-  uint16_t pair[kT * 32 * NPL];                 // (token << 8) | expert
-  uint16_t slot[kT * 32 * NPL];                 // chain slot -> pair (0xffff: none)
-  float zc[kT * 32 * NPL];                      // exact scores of the pairs
+  __align__(16) uint32_t zero[2][32];  // 64 k of +0 (token side) and of -0 (expert side)
+  uint16_t pair[C::kCap];  // (token << 8) | expert
+  uint16_t duo[C::kCap];   // first pair of the duo, kDuoFull when it has a second
+  float zc[C::kCap];       // exact scores of the pairs
 };
+constexpr uint32_t kDuoFull = 0x8000u;
 template <int NPL>
 constexpr size_t batch_smem_bytes() {
   return 1024 + BatchCfg<NPL>::kStages * BatchCfg<NPL>::kStageBytes + sizeof(BatchSmem<NPL>);
 }
 static_assert(batch_smem_bytes<8>() <= 227 * 1024, "one CTA per SM at 256 experts");
+static_assert(3 * (batch_smem_bytes<2>() + 1024) <= 228 * 1024, "three CTAs per SM at 64");
 
 // 16 bytes of shared memory.  The "memory" clobber keeps every such read
 // between the stage's mbarrier wait and its release (both asm statements
@@ -1241,12 +1253,27 @@ __device__ __forceinline__ uint4 lds128(uint32_t addr) {
                : "memory");
   return v;
 }
-// Row r of a 128-byte-swizzled box of 128-byte rows at a 1024-aligned
-// address: the 16-byte chunk q sits at r * 128 + ((q ^ (r & 7)) << 4), i.e.
-// at (base + r * 128 + ((r & 7) << 4)) ^ (q << 4) (bits 4-6 of the row base
-// hold r & 7); swz_row gives the part before the XOR.
-__device__ __forceinline__ uint32_t swz_row(int r) {
-  return static_cast<uint32_t>(r * 128 + ((r & 7) << 4));
+// Descending sort of N keys (N = 2, or 8 by the 19-exchange network of
+// Knuth, The Art of Computer Programming vol. 3, 5.3.4).
+template <int N>
+__device__ __forceinline__ void sort_desc(uint32_t (&k)[N]) {
+  auto ce = [&](int a, int b) {
+    const uint32_t x = max(k[a], k[b]), y = min(k[a], k[b]);
+    k[a] = x;
+    k[b] = y;
+  };
+  if constexpr (N == 2) {
+    ce(0, 1);
+  } else {
+    static_assert(N == 8, "two or eight groups");
+    ce(0, 1); ce(2, 3); ce(4, 5); ce(6, 7);
+    ce(0, 2); ce(1, 3); ce(4, 6); ce(5, 7);
+    ce(1, 2); ce(5, 6); ce(0, 4); ce(3, 7);
+    ce(1, 5); ce(2, 6);
+    ce(1, 4); ce(3, 6);
+    ce(2, 4); ce(3, 5);
+    ce(3, 4);
+  }
 }
 __device__ __forceinline__ void chain8(float& acc, const uint4& a, const uint4& b) {
   fma_lo(acc, a.x, b.x);
@@ -1274,54 +1301,52 @@ __device__ __forceinline__ uint32_t screen_key(float v, int e) {
 }
 
 template <int NPL>
-__global__ void __launch_bounds__(kBatchThreads, BatchCfg<NPL>::kMinCtas)
+__global__ void __launch_bounds__(BatchCfg<NPL>::kThreads, BatchCfg<NPL>::kMinCtas)
     screen_batch_kernel(const __grid_constant__ CUtensorMap map_h,
                         const __grid_constant__ CUtensorMap map_w, float* __restrict__ z,
                         const float* __restrict__ hss, const float* __restrict__ nw, float g,
                         const int32_t* __restrict__ kin, int T, int E, int d, int k_max,
-                        int32_t* __restrict__ ids, float* __restrict__ alpha,
+                        int tpc, int32_t* __restrict__ ids, float* __restrict__ alpha,
                         uint32_t* __restrict__ err) {
   extern __shared__ uint8_t smem_raw[];
   uint8_t* ring = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   using Cf = BatchCfg<NPL>;
-  constexpr int kBatchT = Cf::kT;
-  constexpr int kBatchStages = Cf::kStages;
-  constexpr uint32_t kBatchTokBytes = Cf::kTokBytes;
+  constexpr int kStages = Cf::kStages, kW = Cf::kWarps;
+  constexpr uint32_t kTokBytes = Cf::kTokBytes;
   constexpr int kGroup = Cf::kGroup;
   constexpr uint32_t kStageBytes = Cf::kStageBytes;
   constexpr uint32_t kIdMask = (1u << Cf::kIdBits) - 1u;
-  BatchSmem<NPL>& sm =
-      *reinterpret_cast<BatchSmem<NPL>*>(ring + kBatchStages * kStageBytes);
+  BatchSmem<NPL>& sm = *reinterpret_cast<BatchSmem<NPL>*>(ring + kStages * kStageBytes);
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int t0 = blockIdx.x * kBatchT;
-  const int nt = min(kBatchT, T - t0);
+  const int t0 = blockIdx.x * tpc;  // tpc tokens per CTA (at most kT)
+  const int nt = min(tpc, T - t0);
   const int kcap = k_max < E ? k_max : E;
   if (threadIdx.x == 0) {
-    for (int s = 0; s < kBatchStages; ++s) {
+    for (int s = 0; s < kStages; ++s) {
       mbar_init(&sm.full[s], 1);
-      mbar_init(&sm.empty[s], kBatchCompute / 32);
+      mbar_init(&sm.empty[s], kW);
     }
     sm.abort = 0;
     fence_mbar_init();
   }
+  if (threadIdx.x < 64) sm.zero[threadIdx.x >> 5][lane] = threadIdx.x < 32 ? 0u : 0x80008000u;
   grid_dep_wait();
   grid_dep_launch();
   // ---- 1. screening: candidate masks, kGroup tokens' rounds interleaved ----
-  if (warp < 8) {
+  // warp w takes tokens w, w + kW, ...
+  if (warp < kW) {
     float nwj[NPL];  // the norms of this lane's experts lane + 32 j
 #pragma unroll
     for (int j = 0; j < NPL; ++j) nwj[j] = lane + 32 * j < E ? nw[lane + 32 * j] : 0.f;
-    for (int g0 = 0; g0 < kBatchT / 8; g0 += kGroup) {
+    for (int g0 = warp; g0 < Cf::kT; g0 += kGroup * kW) {
       float zv[kGroup][NPL], hs[kGroup];
       int kt[kGroup];
 #pragma unroll
       for (int i = 0; i < kGroup; ++i) {  // every load of the group first
-        // a warp's last group is partial when kBatchT / 8 is not a multiple
-        // of kGroup
-        const int tl = warp * (kBatchT / 8) + g0 + i;
+        const int tl = g0 + i * kW;
         const int t = t0 + tl;
-        const bool ok = g0 + i < kBatchT / 8 && tl < nt;
+        const bool ok = tl < nt;
         kt[i] = ok ? kin[t] : 1;
         hs[i] = ok ? hss[t] : 0.f;
         const float* zt = z + static_cast<int64_t>(ok ? t : 0) * E;
@@ -1329,15 +1354,15 @@ __global__ void __launch_bounds__(kBatchThreads, BatchCfg<NPL>::kMinCtas)
         for (int j = 0; j < NPL; ++j)
           zv[i][j] = ok && lane + 32 * j < E ? zt[lane + 32 * j] : 0.f;
       }
-      // 32-bit keys: one shuffle per step of the rounds' warp maximum
+      // 32-bit keys, each lane's in descending order: a round is one warp
+      // reduction over the lanes' heads, and the owner of the largest drops it
       uint32_t key[kGroup][NPL], best[kGroup];
       float hi[kGroup][NPL];
       int rounds = 0;
 #pragma unroll
       for (int i = 0; i < kGroup; ++i) {
         if (kt[i] < 1 || kt[i] > kcap) {
-          const int tl = warp * (kBatchT / 8) + g0 + i;
-          if (lane == 0 && g0 + i < kBatchT / 8 && tl < nt) set_err(err, kErrKRange);
+          if (lane == 0 && g0 + i * kW < nt) set_err(err, kErrKRange);
           kt[i] = kt[i] < 1 ? 1 : kcap;
         }
         rounds = max(rounds, kt[i]);
@@ -1355,34 +1380,27 @@ __global__ void __launch_bounds__(kBatchThreads, BatchCfg<NPL>::kMinCtas)
           }
         }
         best[i] = 0u;
+        sort_desc<NPL>(key[i]);
       }
       for (int r = 0; r < rounds; ++r) {
         uint32_t b[kGroup];
 #pragma unroll
-        for (int i = 0; i < kGroup; ++i) {
-          b[i] = key[i][0];
-#pragma unroll
-          for (int j = 1; j < NPL; ++j) b[i] = max(b[i], key[i][j]);
-        }
-#pragma unroll
-        for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-          for (int i = 0; i < kGroup; ++i)
-            b[i] = max(b[i], __shfl_xor_sync(0xffffffffu, b[i], o));
+        for (int i = 0; i < kGroup; ++i) b[i] = __reduce_max_sync(0xffffffffu, key[i][0]);
 #pragma unroll
         for (int i = 0; i < kGroup; ++i) {
           if (r < kt[i]) {
             best[i] = b[i];
+            const bool own = key[i][0] == b[i];
 #pragma unroll
-            for (int j = 0; j < NPL; ++j)
-              if (key[i][j] == b[i]) key[i][j] = 0u;
+            for (int j = 0; j + 1 < NPL; ++j) key[i][j] = own ? key[i][j + 1] : key[i][j];
+            if (own) key[i][NPL - 1] = 0u;
           }
         }
       }
 #pragma unroll
       for (int i = 0; i < kGroup; ++i) {
-        if (g0 + i >= kBatchT / 8) break;  // the next warp's token
-        const int tl = warp * (kBatchT / 8) + g0 + i;
+        const int tl = g0 + i * kW;
+        if (tl >= Cf::kT) break;
         const float L = from_order_bits(best[i] & ~kIdMask);
         int c = 0;
 #pragma unroll
@@ -1399,9 +1417,14 @@ __global__ void __launch_bounds__(kBatchThreads, BatchCfg<NPL>::kMinCtas)
     }
   }
   __syncthreads();
-  if (warp == 0) {  // exclusive prefix of the candidate counts
-    int a = lane < kBatchT ? sm.cnt[lane] : 0;
-    int b = lane + 32 < kBatchT ? sm.cnt[lane + 32] : 0;
+  if (warp < 2) {  // exclusive prefixes: candidate pairs (warp 0), duos (warp 1)
+    int a = lane < Cf::kT ? sm.cnt[lane] : 0;
+    int b = lane + 32 < Cf::kT ? sm.cnt[lane + 32] : 0;
+    if (warp == 1) {
+      a = (a + 1) >> 1;
+      b = (b + 1) >> 1;
+    }
+    int32_t* off = warp == 0 ? sm.off : sm.doff;
     int ia = a, ib = b;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -1413,234 +1436,245 @@ __global__ void __launch_bounds__(kBatchThreads, BatchCfg<NPL>::kMinCtas)
       }
     }
     const int tot_a = __shfl_sync(0xffffffffu, ia, 31);
-    if (lane < kBatchT) sm.off[lane] = ia - a;
-    if (lane + 32 < kBatchT) sm.off[lane + 32] = tot_a + ib - b;
-    if (lane == 31) sm.off[kBatchT] = tot_a + ib;  // the total
+    if (lane < Cf::kT) off[lane] = ia - a;
+    if (lane + 32 < Cf::kT) off[lane + 32] = tot_a + ib - b;
+    if (lane == 31) off[Cf::kT] = tot_a + ib;  // the total
   }
   __syncthreads();
-  if (warp < 8) {  // the (token, expert) pairs in token order, experts ascending
-    for (int i = 0; i < kBatchT / 8; ++i) {
-      const int tl = warp * (kBatchT / 8) + i;
-      const uint32_t below = (1u << lane) - 1u;
-      int pos = sm.off[tl];
-#pragma unroll
-      for (int j = 0; j < NPL; ++j) {
-        const uint32_t m = sm.mask[tl][j];
-        if ((m >> lane) & 1u)
-          sm.pair[pos + __popc(m & below)] = static_cast<uint16_t>((tl << 8) | (lane + 32 * j));
-        pos += __popc(m);
-      }
-    }
-  }
-  __syncthreads();
-  const int npairs = sm.off[kBatchT];
-  // Chain slots: each run of 32 pairs is reordered so that the 8 lanes of a
-  // quarter warp read expert rows of distinct swizzle classes (e & 7): a
-  // 16-byte shared load is served a quarter warp per wavefront, and rows of
-  // one class share a bank group.  The pairs are sorted by class within the
-  // run and dealt to the quarters in turn (sorted position i -> lane
-  // 8 (i % 4) + i / 4).
-  if (warp < 8) {
-    for (int base = warp * 32; base < npairs; base += 8 * 32) {
-      const int idx = base + lane;
-      const bool valid = idx < npairs;
-      const int cls = valid ? (sm.pair[idx] & 7) : 8;
-      int pos = 0;
-#pragma unroll
-      for (int c = 0; c <= 8; ++c) {
-        const uint32_t mc = __ballot_sync(0xffffffffu, cls == c);
-        if (c < cls) pos += __popc(mc);
-        if (c == cls) pos += __popc(mc & ((1u << lane) - 1u));
-      }
-      sm.slot[base + 8 * (pos & 3) + (pos >> 2)] = valid ? static_cast<uint16_t>(idx) : 0xffff;
-    }
-  }
-  __syncthreads();
-  const int nslots = (npairs + 31) & ~31;
-  const int passes = (nslots + kBatchSlots - 1) / kBatchSlots;
   const int nch = d / 64;
-  // ---- 2. the chains ----
-  if (warp == 8) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0, issued = 0, issued_phase = 0;
+  const uint32_t ring_s = smem_addr(ring);
+  int stage = 0;  // ring position of the producer lane and of every compute thread
+  uint32_t phase = 0, issued = 0, issued_phase = 0;
+  // Rounds of consecutive tokens [ta, tb) with at most kCap candidate pairs
+  // (nearly always one round).
+  for (int ta = 0, tb = 0; ta < nt; ta = tb) {
+    const int base_off = sm.off[ta];
+    tb = nt;
+    if (sm.off[nt] - base_off > Cf::kCap) {
+      tb = ta + 1;
+      while (tb < nt && sm.off[tb + 1] - base_off <= Cf::kCap) ++tb;
+    }
+    const int base_duo = sm.doff[ta];
+    const int nduos = sm.doff[tb] - base_duo;
+    if (warp < kW) {  // the (token, expert) pairs in token order, experts ascending
+      for (int tl = ta + warp; tl < tb; tl += kW) {
+        const uint32_t below = (1u << lane) - 1u;
+        const int first = sm.off[tl] - base_off, m = sm.cnt[tl];
+        int pos = first;
+#pragma unroll
+        for (int j = 0; j < NPL; ++j) {
+          const uint32_t m32 = sm.mask[tl][j];
+          if ((m32 >> lane) & 1u)
+            sm.pair[pos + __popc(m32 & below)] =
+                static_cast<uint16_t>((tl << 8) | (lane + 32 * j));
+          pos += __popc(m32);
+        }
+        for (int q = lane; 2 * q < m; q += 32)
+          sm.duo[sm.doff[tl] - base_duo + q] =
+              static_cast<uint16_t>((first + 2 * q) | (2 * q + 1 < m ? kDuoFull : 0u));
+      }
+    }
+    __syncthreads();
+    const int passes = (nduos + Cf::kCompute - 1) / Cf::kCompute;
+    // ---- 2. the chains ----
+    if (warp == kW) {
+      if (lane == 0) {
+        bool ok = true;
+        for (int ps = 0; ps < passes && ok; ++ps) {
+          for (int c = 0; c < nch; ++c) {
+            if (!mbar_wait(&sm.empty[stage], phase ^ 1u, &sm.abort, kBatchWaitNs)) {
+              ok = false;
+              break;
+            }
+            const uint32_t fb = smem_addr(&sm.full[stage]);
+            uint8_t* st = ring + stage * kStageBytes;
+            mbar_arrive_tx(fb, kStageBytes);
+            tma_tile_2d(smem_addr(st), &map_h, c * 64, t0, fb);
+            tma_tile_2d(smem_addr(st + kTokBytes), &map_w, c * 64, 0, fb);
+            issued |= 1u << stage;
+            issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
+            if (++stage == kStages) {
+              stage = 0;
+              phase ^= 1u;
+            }
+          }
+        }
+        if (!ok) {
+          set_err(err, kErrTimeout);
+          sm.abort = 1;
+        }
+        if (sm.abort) {  // every issued copy lands before the CTA exits
+          for (int s = 0; s < kStages; ++s)
+            if (issued & (1u << s))
+              mbar_wait(&sm.full[s], (issued_phase >> s) & 1u, nullptr, kBatchDrainNs);
+        }
+      }
+    } else {
       bool ok = true;
       for (int ps = 0; ps < passes && ok; ++ps) {
-        for (int c = 0; c < nch; ++c) {
-          if (!mbar_wait(&sm.empty[stage], phase ^ 1u, &sm.abort, kBatchWaitNs)) {
-            ok = false;
-            break;
+        // Thread i of a pass advances the chains of duo i: two candidates of
+        // one token, so a step of 8 k reads the token's 16 bytes once and 16
+        // bytes of each expert row.  The rows lie unswizzled, 128 bytes of 64
+        // k each: chunk q of every row starts in the same four banks, so lane
+        // l runs l mod 8 steps behind lane 0 and the eight lanes of a quarter
+        // warp (one shared-memory wavefront) always read eight different
+        // chunks.  The lanes' steps of one chunk therefore span this chunk's
+        // stage and the one before it; before the first and after the last
+        // chunk a lane reads zeros, +0 times -0, which leave every sum as it is.
+        const int i = ps * Cf::kCompute + threadIdx.x;
+        const bool any = __any_sync(0xffffffffu, i < nduos);
+        const uint32_t dv = i < nduos ? sm.duo[i] : 0u;
+        const int p0 = static_cast<int>(dv & (kDuoFull - 1u));
+        const uint32_t q0 = sm.pair[p0];
+        const uint32_t q1 = (dv & kDuoFull) ? sm.pair[p0 + 1] : q0;
+        const uint32_t hrow = (q0 >> 8) * 128u;
+        const uint32_t r0 = kTokBytes + (q0 & 255u) * 128u, r1 = kTokBytes + (q1 & 255u) * 128u;
+        const int l8 = lane & 7;
+        const uint32_t behind = static_cast<uint32_t>(l8) * 16u;
+        const uint32_t zt = smem_addr(sm.zero[0]), ze = smem_addr(sm.zero[1]);
+        float acc0 = 0.f, acc1 = 0.f;
+        uint32_t ph = zt, pa = ze, pb = ze;  // the rows in the stage before
+        int prev = 0;
+        for (int c = 0; c <= nch; ++c) {
+          uint32_t ch = zt, ca = ze, cb = ze;
+          if (c < nch) {
+            if (!__all_sync(0xffffffffu,
+                            mbar_wait(&sm.full[stage], phase, &sm.abort, kBatchWaitNs))) {
+              ok = false;
+              break;
+            }
+            const uint32_t sb = ring_s + stage * kStageBytes;
+            ch = sb + hrow;
+            ca = sb + r0;
+            cb = sb + r1;
           }
-          const uint32_t fb = smem_addr(&sm.full[stage]);
-          uint8_t* st = ring + stage * kStageBytes;
-          mbar_arrive_tx(fb, kStageBytes);
-          tma_tile_2d(smem_addr(st), &map_h, c * 64, t0, fb);
-          tma_tile_2d(smem_addr(st + kBatchTokBytes), &map_w, c * 64, 0, fb);
-          issued |= 1u << stage;
-          issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
-          if (++stage == kBatchStages) {
+          if (any) {
+            // step q: chunk q - l8 of this stage, or 8 + q - l8 of the one before
+            const uint32_t nh = ch - behind, na = ca - behind, nb = cb - behind;
+            const uint32_t oh = ph + 128u - behind, oa = pa + 128u - behind,
+                           ob = pb + 128u - behind;
+            uint4 a = lds128(l8 > 0 ? oh : nh), b0 = lds128(l8 > 0 ? oa : na),
+                  b1 = lds128(l8 > 0 ? ob : nb);
+#pragma unroll
+            for (int q = 0; q < 8; ++q) {
+              uint4 xa, x0, x1;
+              if (q + 1 < 8) {
+                const bool old = q + 1 < l8;
+                xa = lds128((old ? oh : nh) + 16 * (q + 1));
+                x0 = lds128((old ? oa : na) + 16 * (q + 1));
+                x1 = lds128((old ? ob : nb) + 16 * (q + 1));
+              }
+              chain8(acc0, a, b0);
+              chain8(acc1, a, b1);
+              if (q + 1 < 8) {
+                a = xa;
+                b0 = x0;
+                b1 = x1;
+              }
+            }
+            ph = ch;
+            pa = ca;
+            pb = cb;
+          }
+          fence_proxy_async_smem();  // the reads above, before the next TMA fill
+          __syncwarp();
+          if (c > 0 && lane == 0) mbar_arrive_local(smem_addr(&sm.empty[prev]));
+          prev = stage;
+          if (c < nch && ++stage == kStages) {
             stage = 0;
             phase ^= 1u;
           }
         }
+        if (ok && i < nduos) {
+          sm.zc[p0] = acc0;
+          if (dv & kDuoFull) sm.zc[p0 + 1] = acc1;
+        }
       }
-      if (!ok) {
+      if (!ok && lane == 0) {
         set_err(err, kErrTimeout);
         sm.abort = 1;
       }
-      if (sm.abort) {  // every issued copy lands before the CTA exits
-        for (int s = 0; s < kBatchStages; ++s)
-          if (issued & (1u << s))
-            mbar_wait(&sm.full[s], (issued_phase >> s) & 1u, nullptr, kBatchDrainNs);
-      }
     }
-  } else {
-    const uint32_t ring_s = smem_addr(ring);
-    int stage = 0;
-    uint32_t phase = 0;
-    bool ok = true;
-    for (int ps = 0; ps < passes && ok; ++ps) {
-      const int s0 = ps * kBatchSlots + threadIdx.x, s1 = s0 + kBatchCompute;
-      const int p0 = s0 < nslots ? sm.slot[s0] : 0xffff;
-      const int p1 = s1 < nslots ? sm.slot[s1] : 0xffff;
-      const uint32_t q0 = p0 != 0xffff ? sm.pair[p0] : 0u;
-      const uint32_t q1 = p1 != 0xffff ? sm.pair[p1] : 0u;
-      // row bases inside a stage (the swizzle is an XOR on bits 4-6)
-      const uint32_t ta0 = swz_row(q0 >> 8), ea0 = kBatchTokBytes + swz_row(q0 & 255);
-      const uint32_t ta1 = swz_row(q1 >> 8), ea1 = kBatchTokBytes + swz_row(q1 & 255);
-      // the second slot only where a lane of the warp has a pair for it
-      const bool two = __any_sync(0xffffffffu, p1 != 0xffff);
-      float acc0 = 0.f, acc1 = 0.f;
-      for (int c = 0; c < nch; ++c) {
-        if (!__all_sync(0xffffffffu,
-                        mbar_wait(&sm.full[stage], phase, &sm.abort, kBatchWaitNs))) {
-          ok = false;
-          break;
-        }
-        const uint32_t sb = ring_s + stage * kStageBytes;
-        const uint32_t h0 = sb + ta0, w0 = sb + ea0, h1 = sb + ta1, w1 = sb + ea1;
-        if (two) {
-          uint4 a0 = lds128(h0), b0 = lds128(w0), a1 = lds128(h1), b1 = lds128(w1);
-#pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            uint4 na0, nb0, na1, nb1;
-            if (q + 1 < 8) {
-              const uint32_t x = static_cast<uint32_t>((q + 1) << 4);
-              na0 = lds128(h0 ^ x);
-              nb0 = lds128(w0 ^ x);
-              na1 = lds128(h1 ^ x);
-              nb1 = lds128(w1 ^ x);
-            }
-            chain8(acc0, a0, b0);
-            chain8(acc1, a1, b1);
-            if (q + 1 < 8) {
-              a0 = na0;
-              b0 = nb0;
-              a1 = na1;
-              b1 = nb1;
-            }
+    __syncthreads();
+    if (sm.abort) return;
+    // ---- 3. selection over the candidates' exact scores ----
+    // A warp per token: lane l takes candidates l + 32 j, keys as in
+    // select_kernel (score, then the lower expert index); a candidate's rank is
+    // the number of the token's candidates with a larger key, and the k_t
+    // candidates of rank < k_t go to slot rank (the TopK in rank order).
+    if (warp < kW) {
+      for (int tl = ta + warp; tl < tb; tl += kW) {
+        const int t = t0 + tl;
+        const int off = sm.off[tl] - base_off, m = sm.cnt[tl], kt = sm.kt[tl];
+        float* zt = z + static_cast<int64_t>(t) * E;
+        if (m <= 32) {
+          // one candidate per lane, experts ascending with the lanes
+          int e = 0;
+          uint32_t bits = 0u;
+          if (lane < m) {
+            e = sm.pair[off + lane] & 255;
+            const float v = sm.zc[off + lane];
+            zt[e] = v;
+            bits = order_bits(v == 0.0f ? 0.0f : v);
+          }
+          int rank = 0;
+          for (int o = 0; o < m; ++o) {
+            const uint32_t ob = __shfl_sync(0xffffffffu, bits, o);
+            rank += ob > bits || (ob == bits && o < lane);
+          }
+          if (lane < m && rank < kt) {
+            sm.sel_e[warp][rank] = e;
+            sm.sel_z[warp][rank] = from_order_bits(bits);
           }
         } else {
-          uint4 a0 = lds128(h0), b0 = lds128(w0);
+          unsigned long long key[NPL];
+          int ex[NPL], rank[NPL];
 #pragma unroll
-          for (int q = 0; q < 8; ++q) {
-            uint4 na0, nb0;
-            if (q + 1 < 8) {
-              const uint32_t x = static_cast<uint32_t>((q + 1) << 4);
-              na0 = lds128(h0 ^ x);
-              nb0 = lds128(w0 ^ x);
+          for (int j = 0; j < NPL; ++j) {
+            const int idx = lane + 32 * j;
+            key[j] = 0ull;
+            ex[j] = rank[j] = 0;
+            if (idx < m) {
+              ex[j] = sm.pair[off + idx] & 255;
+              const float v = sm.zc[off + idx];
+              zt[ex[j]] = v;
+              key[j] = score_key(v, ex[j]);
             }
-            chain8(acc0, a0, b0);
-            if (q + 1 < 8) {
-              a0 = na0;
-              b0 = nb0;
+          }
+          for (int o = 0; o < m; ++o) {
+            const unsigned long long ko =
+                score_key(sm.zc[off + o], sm.pair[off + o] & 255);  // broadcast reads
+#pragma unroll
+            for (int j = 0; j < NPL; ++j) rank[j] += ko > key[j];
+          }
+#pragma unroll
+          for (int j = 0; j < NPL; ++j) {
+            if (lane + 32 * j < m && rank[j] < kt) {
+              sm.sel_e[warp][rank[j]] = ex[j];
+              sm.sel_z[warp][rank[j]] = from_order_bits(static_cast<uint32_t>(key[j] >> 32));
             }
           }
         }
-        fence_proxy_async_smem();  // the reads above, before the next TMA fill
         __syncwarp();
-        if (lane == 0) mbar_arrive_local(smem_addr(&sm.empty[stage]));
-        if (++stage == kBatchStages) {
-          stage = 0;
-          phase ^= 1u;
+        const float zmax = sm.sel_z[warp][0];
+        const float mine = lane < kt ? expf(sm.sel_z[warp][lane] - zmax) : 0.f;
+        float sel = mine;
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) sel += __shfl_xor_sync(0xffffffffu, sel, o);
+        for (int j = lane; j < k_max; j += 32) {
+          const int64_t o = static_cast<int64_t>(t) * k_max + j;
+          if (j < kt) {
+            ids[o] = sm.sel_e[warp][j];
+            alpha[o] = mine / sel;
+          } else {
+            ids[o] = -1;
+            alpha[o] = 0.f;
+          }
         }
-      }
-      if (ok) {
-        if (p0 != 0xffff) sm.zc[p0] = acc0;
-        if (p1 != 0xffff) sm.zc[p1] = acc1;
+        __syncwarp();
       }
     }
-    if (!ok && lane == 0) {
-      set_err(err, kErrTimeout);
-      sm.abort = 1;
-    }
-  }
-  __syncthreads();
-  if (sm.abort) return;
-  // ---- 3. selection over the candidates' exact scores ----
-  // A warp per token: lane l takes candidates l + 32 j, keys as in
-  // select_kernel (score, then the lower expert index); a candidate's rank is
-  // the number of the token's candidates with a larger key, and the k_t
-  // candidates of rank < k_t go to slot rank (the TopK in rank order).
-  if (warp < 8) {
-    for (int i = 0; i < kBatchT / 8; ++i) {
-      const int tl = warp * (kBatchT / 8) + i;
-      if (tl >= nt) continue;
-      const int t = t0 + tl;
-      const int off = sm.off[tl], m = sm.cnt[tl], kt = sm.kt[tl];
-      const int nj = (m + 31) / 32;  // candidate groups of 32 in use
-      float* zt = z + static_cast<int64_t>(t) * E;
-      unsigned long long key[NPL];
-      int ex[NPL];
-#pragma unroll
-      for (int j = 0; j < NPL; ++j) {
-        const int idx = lane + 32 * j;
-        key[j] = 0ull;
-        ex[j] = 0;
-        if (idx < m) {
-          ex[j] = sm.pair[off + idx] & 255;
-          const float v = sm.zc[off + idx];
-          zt[ex[j]] = v;
-          key[j] = score_key(v, ex[j]);
-        }
-      }
-      // every candidate's key in shared memory (the token's zc slots hold
-      // the scores; the keys are rebuilt from them), then the ranks
-      int rank[NPL];
-#pragma unroll
-      for (int j = 0; j < NPL; ++j) rank[j] = 0;
-      for (int o = 0; o < m; ++o) {
-        const unsigned long long ko =
-            score_key(sm.zc[off + o], sm.pair[off + o] & 255);  // broadcast reads
-#pragma unroll
-        for (int j = 0; j < NPL; ++j)
-          if (j < nj) rank[j] += ko > key[j];
-      }
-#pragma unroll
-      for (int j = 0; j < NPL; ++j) {
-        if (lane + 32 * j < m && rank[j] < kt) {
-          sm.sel_e[warp][rank[j]] = ex[j];
-          sm.sel_z[warp][rank[j]] = from_order_bits(static_cast<uint32_t>(key[j] >> 32));
-        }
-      }
-      __syncwarp();
-      const float zmax = sm.sel_z[warp][0];
-      const float mine = lane < kt ? expf(sm.sel_z[warp][lane] - zmax) : 0.f;
-      float sel = mine;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) sel += __shfl_xor_sync(0xffffffffu, sel, o);
-      for (int j = lane; j < k_max; j += 32) {
-        const int64_t o = static_cast<int64_t>(t) * k_max + j;
-        if (j < kt) {
-          ids[o] = sm.sel_e[warp][j];
-          alpha[o] = mine / sel;
-        } else {
-          ids[o] = -1;
-          alpha[o] = 0.f;
-        }
-      }
-      __syncwarp();
-    }
+    __syncthreads();  // the pair arrays before the next round's
   }
 }
 
@@ -1765,25 +1799,33 @@ cudaError_t launch_router_screen_batch(const CUtensorMap* map_h, const CUtensorM
                                        float* z, const float* hss, const float* nw,
                                        const int32_t* k, int T, int E, int d, int k_max,
                                        int32_t* ids, float* alpha, uint32_t* err,
-                                       cudaStream_t stream) {
+                                       int num_sms, cudaStream_t stream) {
   if (T == 0) return cudaSuccess;
+  if (num_sms < 1) num_sms = 1;
   if (E > 256 || d % 64 != 0 || d < 64 || k_max > 32) return cudaErrorInvalidValue;
   const double u = 1.0 / 16777216.0;
   const double gamma = d * u / (1.0 - d * u);
   // chain bound + tensor-core allowance + the score's own rounding (one K slice)
   const float g = static_cast<float>((gamma + 1.0 / 4096.0 + 2 * u) * (1.0 + 1e-3));
-  auto go = [&](auto kernel, size_t smem, int rows) -> cudaError_t {
+  auto go = [&](auto kernel, size_t smem, int tpc, int threads) -> cudaError_t {
     const cudaError_t e =
         cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    const dim3 grid((T + rows - 1) / rows), block(kBatchThreads);
+    const dim3 grid((T + tpc - 1) / tpc), block(threads);
     return launch_pdl(kernel, grid, block, smem, stream, *map_h, *map_w, z, hss, nw, g, k, T,
-                      E, d, k_max, ids, alpha, err);
+                      E, d, k_max, tpc, ids, alpha, err);
   };
   // map_h's box is screen_batch_token_rows(E) rows high, map_w's
   // screen_batch_expert_rows(E)
-  if (E <= 64) return go(screen_batch_kernel<2>, batch_smem_bytes<2>(), BatchCfg<2>::kT);
-  return go(screen_batch_kernel<8>, batch_smem_bytes<8>(), BatchCfg<8>::kT);
+  if (E <= 64)
+    return go(screen_batch_kernel<2>, batch_smem_bytes<2>(), BatchCfg<2>::kT,
+              BatchCfg<2>::kThreads);
+  // One CTA per SM: whole waves of CTAs, each of as many tokens as that takes
+  // (8192 tokens: 147 CTAs of 56).
+  const int wave = num_sms * BatchCfg<8>::kT;
+  const int slots = (T + wave - 1) / wave * num_sms;
+  const int tpc = ((T + slots - 1) / slots + 7) / 8 * 8;
+  return go(screen_batch_kernel<8>, batch_smem_bytes<8>(), tpc, BatchCfg<8>::kThreads);
 }
 
 int screen_batch_token_rows(int E) { return E <= 64 ? BatchCfg<2>::kT : BatchCfg<8>::kT; }
