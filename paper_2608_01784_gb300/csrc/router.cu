@@ -1722,19 +1722,43 @@ cudaError_t logits_dispatch(const float* h, const float* w, int T, int d, int E,
 cudaError_t logits_dispatch(const __nv_bfloat16* h, const __nv_bfloat16* w, int T,
                             int d, int E, float* z, uint32_t* zw, int nz, uint32_t* err,
                             int num_sms, cudaStream_t s, const L2Prefetch& pf) {
-  const int64_t per_sm = static_cast<int64_t>(T) * E / (num_sms > 0 ? num_sms : 1);
-  // whole rows resident: 16 x 32 tiles, one CTA of 8 warps per SM (2 x 1
-  // chains per thread), for about 300-640 chains per SM (1024 x 64 scores:
-  // 20.8 -> 18.1 us; 8 warps of 2 x 1 instead of 4 of 2 x 2: step -0.6 us;
-  // fewer chains favour the ring kernel's smaller tiles, more chains need a
-  // second wave)
-  using Res = ResCfg<4, 2, 1, 2, 4>;
-  if (per_sm > 300 && per_sm <= 640 && d % kResChunkK == 0 &&
-      d / kResChunkK <= kResMaxChunks && Res::smem(d) <= 227 * 1024)
+  const int sms = num_sms > 0 ? num_sms : 1;
+  const int64_t per_sm = static_cast<int64_t>(T) * E / sms;
+  // Whole rows resident while every CTA of the grid is (one or two per SM, by
+  // their shared memory): a chain then costs little more than its fma latency.
+  // Small tiles first, since few rows are also loaded soonest (score and
+  // selection kernels, us, against the ring kernel): 4 x 16, 32 tokens x 64
+  // experts 15.2 -> 10.6, 64 x 256 16.9 -> 12.1; 8 x 16, 512 x 64 17.6 ->
+  // 16.0; 16 x 32 of 2 x 1 chains per thread, 700 x 64 19.8 -> 18.3, 1024 x
+  // 64 scores 20.8 -> 18.1 alone.  With more CTAs than fit at a time the ring
+  // kernel's smaller tiles win (1500 x 64: 31.7 -> 25.3).
+  using R1 = ResCfg<4, 1, 1, 1, 2>;
+  using R2 = ResCfg<4, 1, 1, 2, 2>;
+  using R3 = ResCfg<4, 2, 1, 2, 4>;
+  auto resident = [&](int bt, int be, size_t smem, int most) {
+    const int64_t ctas = static_cast<int64_t>((T + bt - 1) / bt) * ((E + be - 1) / be);
+    const int fit = static_cast<int>(static_cast<size_t>(227 * 1024) / (smem + 1024));
+    return d % kResChunkK == 0 && d / kResChunkK <= kResMaxChunks &&
+           ctas <= static_cast<int64_t>(sms) * (fit < most ? fit : most);
+  };
+  if (resident(R1::BT, R1::BE, R1::smem(d), 2))
+    return launch_logits_res<4, 1, 1, 1, 2>(h, w, T, d, E, z, zw, nz, err, pf, s);
+  if (resident(R2::BT, R2::BE, R2::smem(d), 2))
+    return launch_logits_res<4, 1, 1, 2, 2>(h, w, T, d, E, z, zw, nz, err, pf, s);
+  if (resident(R3::BT, R3::BE, R3::smem(d), 1))
     return launch_logits_res<4, 2, 1, 2, 4>(h, w, T, d, E, z, zw, nz, err, pf, s);
-  if (per_sm <= 216) return launch_logits_mx<4, 1, 1, 4, 1, 8>(h, w, T, d, E, z, zw, nz, s);
+  // Ring kernel, score and selection kernels in us: 1 x 2 against 1 x 1 tiles
+  // 512 x 64 16.2 / 17.7, 256 x 64 15.8 / 15.4; 4 x 4 tiles of two-warp CTAs
+  // while one warp per scheduler holds every chain, 4096 x 64 42.3 against
+  // 44.7 (2 x 2); 2 x 4 tiles 1536 x 256 59.2 against 63.8; 4 x 4 again 2048 x
+  // 256 67.5 against 72.6.
+  if (per_sm <= 160 || E <= 8)
+    return launch_logits_mx<4, 1, 1, 4, 1, 8>(h, w, T, d, E, z, zw, nz, s);
   if (per_sm <= 1080) return launch_logits_mx<4, 1, 2, 4, 1, 8>(h, w, T, d, E, z, zw, nz, s);
-  if (per_sm <= 4300) return launch_logits_mx<4, 2, 2, 2, 2, 4, 64>(h, w, T, d, E, z, zw, nz, s);
+  if (per_sm <= 1500) return launch_logits_mx<4, 2, 2, 2, 2, 4, 64>(h, w, T, d, E, z, zw, nz, s);
+  if (per_sm > 2048 && per_sm <= 3072 && E > 32)
+    return launch_logits_mx<4, 2, 4, 2, 2, 4, 64>(h, w, T, d, E, z, zw, nz, s);
+  if (per_sm <= 4300) return launch_logits_mx<8, 4, 4, 1, 2, 4, 64>(h, w, T, d, E, z, zw, nz, s);
   if (per_sm <= 10000) return launch_logits_mx<8, 4, 8, 2, 2, 3, 64>(h, w, T, d, E, z, zw, nz, s);
   if (per_sm <= 20000) return launch_logits_mx<8, 4, 4, 2, 2, 3, 64>(h, w, T, d, E, z, zw, nz, s);
   return launch_logits_mx<8, 4, 8, 2, 2, 4>(h, w, T, d, E, z, zw, nz, s);
