@@ -70,7 +70,9 @@ __device__ __forceinline__ int clip(int k, int lo, int hi) {
   return k < lo ? lo : (k > hi ? hi : k);
 }
 
-__device__ __forceinline__ void budget_body(const float* __restrict__ conf1,
+// The counts of sequence s; its error bits and the sum of its counts go to
+// err_bits and sum of thread 0.
+__device__ __forceinline__ void budget_body(int s, const float* __restrict__ conf1,
                                             const float* __restrict__ conf2,
                                             const uint8_t* __restrict__ hist_len,
                                             const uint8_t* __restrict__ masked,
@@ -78,9 +80,8 @@ __device__ __forceinline__ void budget_body(const float* __restrict__ conf1,
                                             const int32_t* __restrict__ seq_off,
                                             const int32_t* __restrict__ active_block,
                                             int T, const AllocArgs& a,
-                                            int32_t* __restrict__ k_out,
-                                            unsigned long long* __restrict__ k_sum,
-                                            uint32_t* __restrict__ err) {
+                                            int32_t* __restrict__ k_out, uint32_t& err_bits,
+                                            unsigned long long& sum) {
   // J_h scores and positions; the role shuffle reuses the same 32 KB as
   // kMaxJ 64-bit sort words
   __shared__ __align__(16) uint64_t s_raw[kMaxJ];
@@ -89,21 +90,10 @@ __device__ __forceinline__ void budget_body(const float* __restrict__ conf1,
   __shared__ int s_nj;
   __shared__ unsigned long long s_sum;
   __shared__ uint32_t s_err;
-  // With one sequence (one CTA) the sum and the error word are stored
-  // outright at the end, so the caller needs no clearing; with several,
-  // the host clears them and each CTA adds its share.
-  const bool sole = gridDim.x == 1;
-  const int s = blockIdx.x;
   const int lo = seq_off[s], hi = seq_off[s + 1];
   if (lo < 0 || hi > T || lo > hi) {  // malformed offsets: touch no count
-    if (threadIdx.x == 0) {
-      if (sole) {
-        if (err) *err = kErrIndex;
-        if (k_sum) *k_sum = 0ull;
-      } else {
-        set_err(err, kErrIndex);
-      }
-    }
+    err_bits = kErrIndex;
+    sum = 0ull;
     return;
   }
   int act = active_block[s];
@@ -220,22 +210,19 @@ __device__ __forceinline__ void budget_body(const float* __restrict__ conf1,
   for (int o = 16; o > 0; o >>= 1) my_sum += __shfl_xor_sync(0xffffffffu, my_sum, o);
   if ((threadIdx.x & 31) == 0) atomicAdd(&s_sum, my_sum);
   __syncthreads();
-  if (threadIdx.x == 0) {
-    if (sole) {
-      if (err) *err = s_err;
-      if (k_sum) *k_sum = s_sum;
-    } else {
-      if (err && s_err) atomicOr(err, s_err);
-      if (k_sum) atomicAdd(k_sum, s_sum);
-    }
-  }
+  err_bits = s_err;
+  sum = s_sum;
+  __syncthreads();  // the shared words before the next sequence's
 }
 
 // defer = 0: waits for the previous kernel before reading anything.
 // defer = 1: launched right behind a kernel that writes none of its inputs
 // (the router scores of the same forward); it runs alongside that kernel and
-// waits for it only before exiting, so that its own completion still implies
-// the completion of everything before it in the stream.
+// waits for it before it adds to the words that kernel may clear and exits,
+// so that its own completion still implies the completion of everything
+// before it in the stream.
+// One CTA per sequence; a single CTA stores the error word and the sum
+// outright, several add their shares to cleared words.
 __global__ void __launch_bounds__(kThreads)
     budget_kernel(const float* __restrict__ conf1, const float* __restrict__ conf2,
                   const uint8_t* __restrict__ hist_len, const uint8_t* __restrict__ masked,
@@ -245,9 +232,20 @@ __global__ void __launch_bounds__(kThreads)
                   uint32_t* __restrict__ err, int defer) {
   if (!defer) grid_dep_wait();
   grid_dep_launch();
-  budget_body(conf1, conf2, hist_len, masked, block_id, seq_off, active_block, T, a, k_out,
-              k_sum, err);
+  uint32_t bits;
+  unsigned long long sum;
+  budget_body(blockIdx.x, conf1, conf2, hist_len, masked, block_id, seq_off, active_block, T, a,
+              k_out, bits, sum);
   if (defer) grid_dep_wait();
+  if (threadIdx.x == 0) {
+    if (gridDim.x == 1) {
+      if (err) *err = bits;
+      if (k_sum) *k_sum = sum;
+    } else {
+      if (err && bits) atomicOr(err, bits);
+      if (k_sum) atomicAdd(k_sum, sum);
+    }
+  }
 }
 
 __global__ void wait_selftest_kernel(uint32_t* err, uint64_t limit_ns) {
@@ -274,8 +272,8 @@ cudaError_t launch_budget(const float* conf1, const float* conf2,
                           unsigned long long* k_sum, uint32_t* err,
                           cudaStream_t stream, bool alongside) {
   if (B <= 0) return cudaSuccess;
-  // programmatic launch when nothing is cleared right before it: a single
-  // sequence, or alongside the router scores (the caller cleared first)
+  // programmatic launch when no memset was issued right before it: a single
+  // sequence, or alongside the router scores
   if (B == 1 || alongside)
     return launch_pdl(budget_kernel, dim3(B), dim3(kThreads), 0, stream, conf1, conf2,
                       hist_len, masked, block_id, seq_off, active_block, T, a, k_out,

@@ -26,6 +26,16 @@ struct WsHeader {
 };
 static_assert(sizeof(WsHeader) == 256, "header is 256 bytes");
 
+// Words that the first kernel of a call clears, so that no memset precedes
+// it: a run of words (the header), and one 32-bit and one 64-bit word of the
+// caller's (nullable).
+struct ZeroWords {
+  uint32_t* words = nullptr;
+  int n = 0;
+  uint32_t* word = nullptr;
+  unsigned long long* sum = nullptr;
+};
+
 constexpr int kTileM = 128;  // rows per grouped-GEMM tile (M of tcgen05.mma)
 
 // ---- programmatic dependent launch -----------------------------------------
@@ -96,6 +106,15 @@ __device__ __forceinline__ float exp_cw(float x) {
   const int k1 = k >> 1;
   const int k2 = k - k1;
   return __fmul_rn(__fmul_rn(p, pow2i(k1)), pow2i(k2));
+}
+
+// Called by one block.
+__device__ __forceinline__ void clear_words(const ZeroWords& z) {
+  for (int i = threadIdx.x; i < z.n; i += blockDim.x) z.words[i] = 0u;
+  if (threadIdx.x == 0) {
+    if (z.word != nullptr) *z.word = 0u;
+    if (z.sum != nullptr) *z.sum = 0ull;
+  }
 }
 
 __device__ __forceinline__ void set_err(uint32_t* err, uint32_t bit) {

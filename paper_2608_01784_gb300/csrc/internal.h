@@ -7,6 +7,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "common.cuh"
+
 namespace rx {
 
 struct AllocArgs {
@@ -21,9 +23,10 @@ struct AllocArgs {
 
 // ---- allocation (budget.cu) -----------------------------------------------
 // alongside: launched right after a kernel that writes none of the inputs
-// (the router scores of the same forward), with err / k_sum already cleared
-// when B > 1; the counts then run next to that kernel, and the budget grid
-// still completes only after it.
+// (the router scores of the same forward) and, when B > 1, itself or the one
+// in front of it clears err / k_sum; the counts then run next to that kernel,
+// and the budget grid adds to the two words and completes only after it.
+// Otherwise, when B > 1, the caller has cleared them.
 cudaError_t launch_budget(const float* conf1, const float* conf2,
                           const uint8_t* hist_len, const uint8_t* masked,
                           const int32_t* block_id, const int32_t* seq_off,
@@ -43,8 +46,8 @@ cudaError_t launch_update_state(const float* conf_new, float* conf1, float* conf
 
 // ---- routing (router.cu) --------------------------------------------------
 // z[T, E] = router scores (sequential fp32 fma chain over the hidden index).
-// The first CTA also clears zero_words[0, n_zero) (nullable): the call's
-// header or error word, so no memset precedes the first kernel.  err
+// The first CTA also clears the zero words (the call's header or error word,
+// the allocation's outputs), so no memset precedes the first kernel.  err
 // (nullable) receives kErrTimeout if a bounded wait of a kernel expires.
 // pf (optional): bytes the score kernel hands to the L2 as bulk prefetches
 // while it computes (the next kernels' weights; HBM is otherwise idle then).
@@ -54,16 +57,16 @@ struct L2Prefetch {
 };
 cudaError_t launch_router_logits(int dtype, const void* hidden,
                                  const void* w_router, int T, int d, int E,
-                                 float* z, uint32_t* zero_words, int n_zero,
-                                 uint32_t* err, int num_sms, cudaStream_t stream,
+                                 float* z, const ZeroWords& zero, uint32_t* err,
+                                 int num_sms, cudaStream_t stream,
                                  const L2Prefetch& pf = L2Prefetch{});
 // Screened routing (bf16, renormalised weights): nw[e] = ||w_e||_2 rounded up
-// (first kernel of the forward; clears zero_words like the score kernels);
+// (first kernel of the forward; clears the zero words like the score kernels);
 // then, from the tensor-core score slices z[s][t][e] (s < k_splits), the
 // exact TopK, alpha and ids, with the canonical chain recomputed for every
 // expert that could be selected (written back into z's first slice).
 cudaError_t launch_router_wnorm(const __nv_bfloat16* w, int E, int d, float* nw,
-                                uint32_t* zero_words, int n_zero, cudaStream_t stream);
+                                const ZeroWords& zero, cudaStream_t stream);
 cudaError_t launch_router_screen_select(const __nv_bfloat16* h, const __nv_bfloat16* w,
                                         float* z, int k_splits, int64_t split_stride,
                                         const float* nw, const int32_t* k, int T, int E,

@@ -227,7 +227,9 @@ rx::AllocArgs alloc_args(const reflex_alloc_params* p) {
 
 // The error word and the pair sum are stored outright by a single-sequence
 // count kernel; with several sequences each CTA adds its share to cleared
-// words, and so does every warp of the score rules' selection.
+// words, and so does every warp of the score rules' selection.  This clears
+// them ahead of counts that have no first kernel of the ROUTE stage in front
+// of them, which clears them otherwise.
 cudaError_t clear_alloc_outputs(const AllocCall& c, cudaStream_t s) {
   if (c.B <= 1 && c.a.count_rule == REFLEX_RULE_REFLEX) return cudaSuccess;
   if (c.err) {
@@ -429,7 +431,16 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
   void* ash = shared_inter ? ws + L.ash : nullptr;
   void* ysh = shared_inter ? ws + L.ysh : nullptr;
 
-  if (ac != nullptr) RX_CUDA(clear_alloc_outputs(*ac, s));
+  // words the first kernel of the ROUTE stage clears: the header (error word,
+  // totals), and what the counts' CTAs or warps add to (two memsets in front
+  // of it cost an 8-sequence step 3 us)
+  rx::ZeroWords zero;
+  zero.words = reinterpret_cast<uint32_t*>(hdr);
+  zero.n = static_cast<int>(sizeof(WsHeader) / 4);
+  if (ac != nullptr && (ac->B > 1 || ac->a.count_rule != REFLEX_RULE_REFLEX)) {
+    zero.word = ac->err;
+    zero.sum = ac->k_sum;
+  }
   // bf16 with renormalised weights, many experts and many scores: tensor-
   // core scores screen the experts and only those that could be selected get
   // the canonical chain (router.cu).  The recheck costs about as much per
@@ -464,8 +475,7 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
     float* nw = reinterpret_cast<float*>(ws + L.wnorm);
     float* hss = reinterpret_cast<float*>(ws + L.tnorm);
     RX_CUDA(rx::launch_router_wnorm(static_cast<const __nv_bfloat16*>(w_router), E, d, nw,
-                                    reinterpret_cast<uint32_t*>(hdr),
-                                    static_cast<int>(sizeof(WsHeader) / 4), s));
+                                    zero, s));
     rx::GroupRows rows{nullptr, nullptr, nullptr, nullptr, 1, T, T};
     rx::TcGemmArgs sa{&mh, &mw, d, E, 0, 0, rows, nullptr, E, err, sms};
     RX_CUDA(rx::launch_scores_tc(sa, sbn, 1, z, static_cast<int64_t>(T) * E, E, true, s, hss));
@@ -483,8 +493,7 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
     // reads and writes nothing it touches, so it runs beside it, and so does
     // the count kernel of reflex_step
     RX_CUDA(rx::launch_router_wnorm(static_cast<const __nv_bfloat16*>(w_router), E, d, nw,
-                                    reinterpret_cast<uint32_t*>(hdr),
-                                    static_cast<int>(sizeof(WsHeader) / 4), s));
+                                    zero, s));
     rx::GroupRows rows{nullptr, nullptr, nullptr, nullptr, 1, T, T};
     rx::TcGemmArgs sa{&mh, &mw, d, E, 0, 0, rows, nullptr, E, err, sms};
     RX_CUDA(rx::launch_scores_tc(sa, bn, ks, z, zs, E, true, s));
@@ -510,9 +519,8 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
       pf.base = w_gate_up;
       pf.bytes = (wbytes < kRouterL2Prefetch ? wbytes : kRouterL2Prefetch) & ~uint64_t{4095};
     }
-    RX_CUDA(rx::launch_router_logits(dtype, hidden, w_router, T, d, E, z,
-                                     reinterpret_cast<uint32_t*>(hdr),
-                                     static_cast<int>(sizeof(WsHeader) / 4), err, sms, s, pf));
+    RX_CUDA(rx::launch_router_logits(dtype, hidden, w_router, T, d, E, z, zero,
+                                     err, sms, s, pf));
     if (rule) {
       // k = ac->k_out: the selection writes the counts it derives
       RX_CUDA(rx::launch_router_select_rule(z, T, E, ac->a.k_max < k_max ? ac->a.k_max : k_max,
@@ -527,6 +535,7 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
                                        I32(L.ids), alpha, err, s));
     }
   } else if (ac != nullptr) {
+    RX_CUDA(clear_alloc_outputs(*ac, s));
     RX_CUDA(launch_alloc(*ac, T, s, false));
   }
   if (stages & REFLEX_STAGE_DISPATCH) {

@@ -89,7 +89,7 @@ extern "C" int reflex_route_noalloc(int32_t dtype, const void* hidden,
   // call can set a bit in it (a 4-byte memset allocates nothing)
   if (err != nullptr && cudaMemsetAsync(err, 0, sizeof(uint32_t), s) != cudaSuccess)
     return REFLEX_ECUDA;
-  if (rx::launch_router_logits(dtype, hidden, w_router, T, d, E, z, nullptr, 0, err, sms,
+  if (rx::launch_router_logits(dtype, hidden, w_router, T, d, E, z, rx::ZeroWords{}, err, sms,
                                s) != cudaSuccess)
     return REFLEX_ECUDA;
   if (rx::launch_router_select(z, k, T, E, k_max, (flags & REFLEX_FLAG_RENORM_TOPK) != 0,
