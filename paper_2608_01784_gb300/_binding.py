@@ -148,7 +148,9 @@ def _ptr(x) -> int | None:
 def _stream(stream) -> int | None:
     if stream is None:
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        # the handle alone: building torch's Stream object takes 2.9 us, more
+        # than a kernel launch
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
