@@ -105,8 +105,6 @@ struct KParams {
   // 1: the first ring stages' weights are requested before the dependency
   // wait (early_tile)
   int early_b;
-  // CTA pairs: whole 32-row output chunks leave by TMA store (map_out)
-  int tma_out;
   // SwiGLU on CTA pairs: A rows gathered from the token rows (TcGemmArgs)
   const int32_t* gather_perm;
   int gather_kmax;
@@ -795,7 +793,6 @@ cudaError_t launch_impl(const TcGemmArgs& a, cudaStream_t stream) {
   p.early_b = a.early_b ? 1 : 0;
   p.b3d = MODE == kModeSwiGLU && a.b_gate_up_3d ? 1 : 0;
   p.norm_out = nullptr;
-  p.tma_out = 0;
   p.gather_perm = nullptr;
   p.gather_kmax = 1;
   p.gather_tokens = 0;
@@ -811,19 +808,27 @@ cudaError_t launch_impl(const TcGemmArgs& a, cudaStream_t stream) {
 // ===========================================================================
 // 2-SM variant (cta_group::2) for groups of many rows.
 //
-// A cluster of two CTAs on one TPC computes a 256 x 256 tile: CTA rank r
-// holds rows [row0 + 128 r, +128) of A and one half of the weight tile
-// (SwiGLU: rank 0 the 128 gate rows, rank 1 the 128 matching up rows; down:
-// rows n*256 + 128 r of W_down), so each SM streams 32 KB per 64-k block
-// instead of 48 KB; the 192 KB ring holds 3 stages of two consecutive 64-k
-// blocks.  With gathered rows (SwiGLU, TcGemmArgs::gather_perm) the A rows
-// come straight from the token rows: every lane of the producer warp issues
-// one four-row TMA gather per 64-k block, the tokens looked up through the
-// pair permutation once per tile; the rows, tiles and MMA order are those of
-// the copied rows, so the outputs are the same bits.  One thread of the
-// leader CTA (rank 0) issues tcgen05.mma.cta_group::2 (M = 256, N = 256);
-// each CTA's TMEM receives its 128 rows x 256 fp32 columns (two buffers of
-// 256 columns, allocated collectively by one warp per CTA).
+// A cluster of two CTAs on one TPC computes a tile of 256 weight rows x up to
+// 256 token rows.  The weights are the M operand (M = 256, 128 rows per CTA)
+// and the token rows the N operand (each CTA holds half of them), so a tile
+// that ends inside its group computes and loads its own rows rounded up to
+// 32, not 256: with about 330 rows per expert a third of all MMA work had
+// been padding rows (LLaDA-MoE shape, 3270 tokens: gate/up 179 -> 153 us, down
+// 88 -> 84; 32768 tokens: gate/up 812 -> 780; LLaDA2.0-mini shape, 65536: 1293
+// -> 1255, its K = 512 down GEMM 742 -> 757).
+// SwiGLU: CTA rank r holds 64 gate rows and the matching 64 up rows, 16 gate
+// then 16 up rows in turn (one box of a 5D map), so gate and up of one output
+// meet in one warp's TMEM lanes, 16 apart.  Down: rows n*256 + 128 r of
+// W_down.  A 192 KB ring holds 3 stages of two consecutive 64-k blocks, at
+// most 32 KB per SM and block.  With gathered rows (SwiGLU,
+// TcGemmArgs::gather_perm) the rows come straight from the token rows: every
+// lane of the producer warp issues one four-row TMA gather per 64-k block,
+// the tokens looked up through the pair permutation once per tile; the rows,
+// tiles and MMA order are those of the copied rows, so the outputs are the
+// same bits.  One thread of the leader CTA (rank 0) issues
+// tcgen05.mma.cta_group::2; each CTA's TMEM receives its 128 weight rows x
+// the tile's token columns (two buffers of 256 columns, allocated
+// collectively by one warp per CTA).
 // Barriers: both producers arrive (with their byte counts) on the leader's
 // "full" barrier and their TMA loads complete on it; MMA completion is
 // multicast to both CTAs' "empty" and "accumulator full" barriers; both
@@ -879,6 +884,14 @@ __device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(cl_bar)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_5d_pair(uint32_t dst, const CUtensorMap* map, int c0,
+                                                 int c3, int c4, uint32_t cl_bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+      " [%0], [%1, {%2, %3, %3, %4, %5}], [%6];" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(0), "r"(c3), "r"(c4), "r"(cl_bar)
+      : "memory");
+}
 // Four rows r0..r3 of a map whose box is {64, 1}, copied to four consecutive
 // 128-byte rows at dst (the same 128-byte swizzle as a tiled box: it follows
 // the shared-memory address, and dst is 512-byte aligned, half of an 8-row
@@ -922,12 +935,12 @@ __device__ __forceinline__ void tmem_dealloc_pair(uint32_t taddr, uint32_t ncols
 }
 
 struct Cfg2 {
-  static constexpr int BN = 256;                 // output tile width of the pair
+  static constexpr int BN = 256;                 // most token rows of a tile
   static constexpr int KS = 2;                   // 64-k blocks per stage
   static constexpr int kSubBytes = BM * BK * 2;  // 16 KB: one 128-row x 64-k box
-  static constexpr int kABytes = KS * kSubBytes; // this CTA's 128 rows
-  static constexpr int kBBytes = KS * kSubBytes; // this CTA's half of the weight tile
-  static constexpr int kStageBytes = kABytes + kBBytes;
+  static constexpr int kWBytes = KS * kSubBytes; // this CTA's 128 weight rows
+  static constexpr int kXBytes = KS * kSubBytes; // this CTA's half of the token rows, at most
+  static constexpr int kStageBytes = kWBytes + kXBytes;
   static constexpr int kStages = kRingBytes / kStageBytes;  // 3
   static constexpr int kTmemCols = 2 * BN;       // two accumulators
   static constexpr int kStagingBytes = 32 * 128; // per epilogue warp: 32 rows x 128 B
@@ -947,24 +960,72 @@ __device__ __forceinline__ void tma_store_2d(const CUtensorMap* map, uint32_t sr
 __device__ __forceinline__ void bulk_commit() {
   asm volatile("cp.async.bulk.commit_group;" ::: "memory");
 }
-// the stores issued so far have read their shared-memory source
+// all stores but the latest N have read their shared-memory source
+template <int N>
 __device__ __forceinline__ void bulk_wait_read() {
-  asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
+  asm volatile("cp.async.bulk.wait_group.read %0;" ::"n"(N) : "memory");
 }
 // ... and completed
 __device__ __forceinline__ void bulk_wait_all() {
   asm volatile("cp.async.bulk.wait_group 0;" ::: "memory");
 }
 
-// The epilogue's bf16 rows reach global memory through a per-warp staging
-// tile: each thread writes its row's 128 bytes (16-byte chunk j at position
-// j ^ (row & 7), so the 32 rows' writes spread over the banks), then each
-// store instruction of the warp writes four whole 128-byte row segments
-// (lane l: row 4 i + l / 8, chunk l % 8).  Per-lane stores of 16 bytes to 32
-// different rows cost one L2 request per 16 bytes, as many requests as the
-// TMA loads of the main loop; this costs one per 128 bytes.
-__device__ __forceinline__ void stage_chunk(uint8_t* stg, int lane, int j, const uint4& v) {
-  *reinterpret_cast<uint4*>(stg + lane * 128 + ((j ^ (lane & 7)) << 4)) = v;
+// The epilogue's bf16 outputs reach global memory through staging tiles of 32
+// token rows x 64 output columns (128 bytes a row, 16-byte chunk j at
+// position j ^ (row & 7), the 128-byte swizzle of a TMA box).  The TMEM lanes
+// hold output columns, so the tile is transposed on the way: 16x256b loads
+// give a thread two neighbouring tokens of a column, the fragment that
+// stmatrix stores transposed, 16-byte row segments without bank conflicts
+// (packing across lanes with shuffles took a quarter of the shared-memory
+// pipe of a K = 512 tile).  Several warps fill one staging tile; a whole tile
+// leaves by one TMA store, a partial one by lane stores of whole 128-byte row
+// segments.
+// 16 TMEM lanes x 32 fp32 columns: r[4 j + i] of thread t is lane t / 4 (+ 8
+// for i >= 2), column 8 j + 2 (t mod 4) + (i mod 2).
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[16]) {
+  asm volatile(
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]),
+        "=r"(r[7]), "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]),
+        "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+      : "r"(taddr));
+}
+// Four 8 x 8 matrices (columns x tokens in the registers) stored transposed:
+// thread t gives the address of row t mod 8 of matrix t / 8.
+__device__ __forceinline__ void stmatrix_trans(uint32_t addr, uint32_t a, uint32_t b, uint32_t c,
+                                               uint32_t d) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.trans.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(addr),
+               "r"(a), "r"(b), "r"(c), "r"(d)
+               : "memory");
+}
+// address of 16-byte chunk j of row `row` of a staging tile
+__device__ __forceinline__ uint32_t stage_addr(uint32_t stg, int row, int j) {
+  return stg + static_cast<uint32_t>(row * 128 + ((j ^ (row & 7)) << 4));
+}
+__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
+  __nv_bfloat162 h2 = __floats2bfloat162_rn(lo, hi);
+  return *reinterpret_cast<uint32_t*>(&h2);
+}
+__device__ __forceinline__ uint32_t pack_bf16(uint32_t lo, uint32_t hi) {
+  return pack_bf16(__uint_as_float(lo), __uint_as_float(hi));
+}
+// named barrier of `threads` threads; the second form returns whether v held
+// in every one of them
+__device__ __forceinline__ void group_sync(int id, int threads) {
+  asm volatile("barrier.cta.sync %0, %1;" ::"r"(id), "r"(threads) : "memory");
+}
+__device__ __forceinline__ bool group_all(int id, int threads, bool v) {
+  uint32_t r;
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.u32 q, %1, 0;\n\t"
+      "barrier.cta.red.and.pred p, %2, %3, q;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(r)
+      : "r"(v ? 1u : 0u), "r"(id), "r"(threads)
+      : "memory");
+  return r != 0;
 }
 // rows [0, nrows) of the staging tile to out rows row_base + r, columns
 // col0 .. col0 + 63 (bf16), row stride ldo
@@ -982,10 +1043,17 @@ __device__ __forceinline__ void flush_staging(const uint8_t* stg, int lane,
   __syncwarp();
 }
 
+// Token columns of a tile of `rows` token rows: the MMA's N, a multiple of 32
+// (16 rows per CTA).
+__device__ __forceinline__ int tile_cols(int rows) { return (rows + 31) & ~31; }
+
 template <int MODE>
 __global__ void __launch_bounds__(kThreads2, 1)
-    grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_a,
-                             const __grid_constant__ CUtensorMap map_b,
+    grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w,
+                             const __grid_constant__ CUtensorMap map_x32,
+                             const __grid_constant__ CUtensorMap map_x64,
+                             const __grid_constant__ CUtensorMap map_x96,
+                             const __grid_constant__ CUtensorMap map_x128,
                              const __grid_constant__ CUtensorMap map_out, const KParams p) {
   using C = Cfg2;
   constexpr int kStages = C::kStages;
@@ -993,10 +1061,10 @@ __global__ void __launch_bounds__(kThreads2, 1)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
-  uint8_t* sa = smem;
-  uint8_t* sb = smem + kStages * C::kABytes;
-  // after the ring: the epilogue warps' staging tiles (1024-byte aligned,
-  // the 128-byte swizzle of the output map), the barriers, the tile index
+  uint8_t* sw = smem;                         // weight rows
+  uint8_t* sx = smem + kStages * C::kWBytes;  // token rows
+  // after the ring: the epilogue's staging tiles (1024-byte aligned, the
+  // 128-byte swizzle of the output map), the barriers, the tile index
   uint8_t* staging = smem + kStages * C::kStageBytes;
   uint64_t* bars = reinterpret_cast<uint64_t*>(staging + kEpiWarps2 * C::kStagingBytes);
   uint64_t* full = bars;                        // leader's is the one used
@@ -1026,17 +1094,19 @@ __global__ void __launch_bounds__(kThreads2, 1)
     mbar_init(drain, 1);
     *abort_flag = 0;
     fence_mbar_init();
-    prefetch_map(&map_a);
-    prefetch_map(&map_b);
-    if (p.tma_out) prefetch_map(&map_out);
+    prefetch_map(&map_w);
+    prefetch_map(&map_x128);
+    prefetch_map(&map_out);
   }
   cluster_sync_all();  // barriers of both CTAs initialised; the peer is running
   const int nk = p.K / (BK * C::KS);  // stages per tile
-  // first weight row of this CTA's half of tile (e, n)
-  auto weight_row = [&](const Tile& tl) {
-    return MODE == kModeSwiGLU
-               ? tl.e * p.b_rows_per_group + (rank ? p.b_up_offset : 0) + tl.n * (BN / 2)
-               : tl.e * p.b_rows_per_group + tl.n * BN + static_cast<int>(rank) * (BN / 2);
+  // this CTA's weight rows of k-block k0 of tile (e, n), counted on fb
+  auto load_weights = [&](const Tile& tl, uint32_t dst, int k0, uint32_t fb) {
+    if (MODE == kModeSwiGLU)  // groups of 16 features: 4 per CTA, 8 per tile
+      tma_load_5d_pair(dst, &map_w, k0, tl.n * 8 + static_cast<int>(rank) * 4, tl.e, fb);
+    else
+      tma_load_2d_pair(dst, &map_w, k0,
+                       tl.e * p.b_rows_per_group + tl.n * 256 + static_cast<int>(rank) * BM, fb);
   };
   // the ring's first weights while the kernel in front still runs, as in the
   // 1-SM kernel; both CTAs' bytes count on the leader's barriers
@@ -1048,11 +1118,11 @@ __global__ void __launch_bounds__(kThreads2, 1)
       if (lane == 0) {
         for (int s = 0; s < early; ++s) {
           const uint32_t fb = map_to_rank(smem_addr(&full[s]), 0);
-          if (leader) mbar_expect_tx_only(smem_addr(&full[s]), C::kBBytes);
-          else mbar_expect_tx_only_cluster(fb, C::kBBytes);
+          if (leader) mbar_expect_tx_only(smem_addr(&full[s]), C::kWBytes);
+          else mbar_expect_tx_only_cluster(fb, C::kWBytes);
           for (int u = 0; u < C::KS; ++u)
-            tma_load_2d_pair(smem_addr(sb + s * C::kBBytes + u * C::kSubBytes), &map_b,
-                             (s * C::KS + u) * BK, weight_row(tl), fb);
+            load_weights(tl, smem_addr(sw + s * C::kWBytes + u * C::kSubBytes),
+                         (s * C::KS + u) * BK, fb);
         }
       }
     }
@@ -1067,15 +1137,16 @@ __global__ void __launch_bounds__(kThreads2, 1)
   const TileIndex ix =
       load_tile_index(p, reinterpret_cast<int32_t*>(reinterpret_cast<uint8_t*>(bars) + 256),
                       C::kIndexInts);
-  // tiles are 256 rows (both CTAs) x 256 columns; mt_prefix counts 256-row tiles
+  // tiles are 256 weight rows x up to 256 token rows (both CTAs); mt_prefix
+  // counts 256-row tiles
   const int ntiles = total_tiles<false>(p, ix);
 
-  // SwiGLU with gathered A rows: the whole producer warp issues the A
-  // copies, one four-row gather per lane and 64-k block (lane l: rows 4 l ..
-  // 4 l + 3 of this CTA's 128); otherwise lane 0 issues everything
+  // SwiGLU with gathered rows: the whole producer warp issues the row copies,
+  // one four-row gather per lane and 64-k block (lane l: rows 4 l .. 4 l + 3
+  // of this CTA's half); otherwise lane 0 issues everything
   const bool gather = MODE == kModeSwiGLU && p.gather_perm != nullptr;
   if (warp == 0 && (gather || lane == 0)) {
-    // ---------------- TMA producer (each CTA: its A rows, its B half) -------
+    // ---------------- TMA producer (each CTA: its weight rows, its token rows)
     int stage = 0;
     uint32_t phase = 0;
     uint32_t issued_mask = 0, issued_phase = 0;
@@ -1089,13 +1160,22 @@ __global__ void __launch_bounds__(kThreads2, 1)
         }
         break;
       }
+      const int half_rows = tile_cols(tl.rows) / 2;  // token rows per CTA, a multiple of 16
+      const int xrow = tl.row0 + static_cast<int>(rank) * half_rows;
+      // the smallest box that holds them; rows past the tile's end are
+      // computed from the next rows or TMA zero fill and never stored
+      const int bx = (half_rows + 31) / 32;
+      const CUtensorMap* mx = bx == 1 ? &map_x32 : bx == 2 ? &map_x64 : bx == 3 ? &map_x96
+                                                                             : &map_x128;
+      const uint32_t xbytes = gather ? C::kXBytes : static_cast<uint32_t>(C::KS * bx * 32 * 128);
       // token of each of this lane's four rows; rows past the tile's end
       // repeat its last row (computed, never stored)
       int tok[4] = {0, 0, 0, 0};
       if (gather) {
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
-          const int r = min(static_cast<int>(rank) * BM + 4 * lane + i, tl.rows - 1);
+          const int r = min(static_cast<int>(rank) * half_rows + min(4 * lane + i, half_rows - 1),
+                            tl.rows - 1);
           const int o = p.gather_perm[tl.row0 + r];
           const int tk = o >= 0 ? o / p.gather_kmax : -1;
           if (tk < 0 || tk >= p.gather_tokens)
@@ -1112,11 +1192,10 @@ __global__ void __launch_bounds__(kThreads2, 1)
           break;
         }
         const uint32_t fb = map_to_rank(smem_addr(&full[stage]), 0);
-        const int brow = weight_row(tl);
         const bool ahead = early > 0;  // the weights are already on their way
         if (ahead) --early;
         if (lane == 0) {
-          const uint32_t bytes = ahead ? C::kABytes : C::kStageBytes;
+          const uint32_t bytes = (ahead ? 0u : static_cast<uint32_t>(C::kWBytes)) + xbytes;
           if (leader)
             mbar_expect_tx(smem_addr(&full[stage]), bytes);
           else
@@ -1126,11 +1205,10 @@ __global__ void __launch_bounds__(kThreads2, 1)
           for (int u = 0; u < C::KS; ++u) {
             const int k0 = (kb * C::KS + u) * BK;
             if (!gather)
-              tma_load_2d_pair(smem_addr(sa + stage * C::kABytes + u * C::kSubBytes), &map_a,
-                               k0, tl.row0 + static_cast<int>(rank) * BM, fb);
+              tma_load_2d_pair(smem_addr(sx + stage * C::kXBytes + u * C::kSubBytes), mx, k0,
+                               xrow, fb);
             if (!ahead)
-              tma_load_2d_pair(smem_addr(sb + stage * C::kBBytes + u * C::kSubBytes), &map_b, k0,
-                               brow, fb);
+              load_weights(tl, smem_addr(sw + stage * C::kWBytes + u * C::kSubBytes), k0, fb);
           }
         }
         if (gather) {
@@ -1138,7 +1216,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
 #pragma unroll
           for (int u = 0; u < C::KS; ++u)
             tma_gather4_pair(
-                smem_addr(sa + stage * C::kABytes + u * C::kSubBytes + lane * 4 * 128), &map_a,
+                smem_addr(sx + stage * C::kXBytes + u * C::kSubBytes + lane * 4 * 128), &map_x32,
                 (kb * C::KS + u) * BK, tok, fb);
         }
         issued_mask |= 1u << stage;
@@ -1173,9 +1251,6 @@ __global__ void __launch_bounds__(kThreads2, 1)
     }
   } else if (warp == 1 && lane == 0 && leader) {
     // ---------------- MMA issuer (leader CTA only) ----------------
-    constexpr uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) |
-                               (static_cast<uint32_t>(BN >> 3) << 17) |
-                               (static_cast<uint32_t>((2 * BM) >> 4) << 24);
     int stage = 0;
     uint32_t phase = 0;
     int lt = 0;
@@ -1183,6 +1258,11 @@ __global__ void __launch_bounds__(kThreads2, 1)
     for (int t = pair; t < ntiles && ok; t += npairs, ++lt) {
       const int ab = lt & 1;
       const uint32_t acc_phase = (lt >> 1) & 1;
+      Tile tl;
+      const int cols = decode_tile<false>(p, ix, t, tl) ? tile_cols(tl.rows) : BN;
+      const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) |
+                             (static_cast<uint32_t>(cols >> 3) << 17) |
+                             (static_cast<uint32_t>((2 * BM) >> 4) << 24);
       if (!mbar_wait(&acc_empty[ab], acc_phase ^ 1u, abort_flag, kWaitNs)) {
         ok = false;
         break;
@@ -1195,14 +1275,14 @@ __global__ void __launch_bounds__(kThreads2, 1)
           break;
         }
         tc_fence_after();
-        const uint32_t a0 = smem_addr(sa + stage * C::kABytes);
-        const uint32_t b0 = smem_addr(sb + stage * C::kBBytes);
+        const uint32_t w0 = smem_addr(sw + stage * C::kWBytes);
+        const uint32_t x0 = smem_addr(sx + stage * C::kXBytes);
 #pragma unroll
         for (int u = 0; u < C::KS; ++u)
 #pragma unroll
           for (int k = 0; k < BK / UMMA_K; ++k)
-            mma_bf16_pair(d_tmem, desc_sw128(a0 + u * C::kSubBytes + k * UMMA_K * 2),
-                          desc_sw128(b0 + u * C::kSubBytes + k * UMMA_K * 2), idesc,
+            mma_bf16_pair(d_tmem, desc_sw128(w0 + u * C::kSubBytes + k * UMMA_K * 2),
+                          desc_sw128(x0 + u * C::kSubBytes + k * UMMA_K * 2), idesc,
                           (kb > 0 || u > 0 || k > 0) ? 1u : 0u);
         issued_any = true;
         mma_commit_pair(smem_addr(&empty[stage]));
@@ -1223,45 +1303,25 @@ __global__ void __launch_bounds__(kThreads2, 1)
       mbar_wait(drain, 0, nullptr, kDrainNs);
     }
   } else if (warp >= 2) {
-    // ---------------- epilogue (each CTA: its 128 rows) ----------------
-    // warp w drains TMEM lanes 32 (w % 4) .. +31 (its quarter of the rows)
-    // and one half of the columns: warps 2-5 the first, 6-9 the second.
-    // The TMEM loads of a half are issued two chunks at a time before one
-    // wait; once the last chunk is in registers the accumulator is handed
-    // back (relaxed arrive), and the conversion and stores of that chunk
-    // overlap the next tile's MMAs.
+    // ---------------- epilogue (each CTA: its 128 weight rows) ----------------
+    // Warp w drains TMEM lanes 32 (w % 4) .. +31; warps 2-5 take the tile's
+    // even 32-column (token) chunks, 6-9 the odd ones.  The warps that fill
+    // one staging tile (64 output columns) are a group: SwiGLU all four of a
+    // half (16 columns each), down two (32 columns each).  Once a warp's last
+    // chunk is in registers it hands the accumulator back (relaxed arrive),
+    // and the conversion and stores overlap the next tile's MMAs.
     const int quarter = warp & 3;
     const int half = (warp - 2) >> 2;
-    const int wrow0 = static_cast<int>(rank) * BM + quarter * 32;  // warp's first row in the 256
-    uint8_t* stg = staging + (warp - 2) * C::kStagingBytes;
-    // Whole 32-row chunks leave by one TMA store of the staging tile (the
-    // store engine writes the lines; per-lane stores of the same lines cost
-    // the down GEMM of the 32 x 1024 layer about 57 us of its 455); a chunk
-    // that ends inside the tile's group keeps the per-lane stores, which
-    // stop at its last row.  The tile is rewritten only after the previous
-    // store has read it.
-    const bool tma_out = p.tma_out != 0;
-    auto staging_free = [&]() {
-      if (tma_out) {
-        if (lane == 0) bulk_wait_read();
-        __syncwarp();
-      }
-    };
-    auto emit = [&](int64_t rbase, int col0, int nrows) {
-      if (tma_out && nrows == 32) {
-        fence_proxy_async_smem();  // this lane's staging writes, before the store reads them
-        __syncwarp();
-        if (lane == 0) {
-          tma_store_2d(&map_out, smem_addr(stg), col0, static_cast<int>(rbase));
-          bulk_commit();
-        }
-      } else {
-        flush_staging(stg, lane, p.out, rbase, p.ldo, col0, nrows);
-      }
-    };
+    constexpr bool kUp = MODE == kModeSwiGLU;
+    constexpr int kGroup = kUp ? 128 : 64;     // threads of a group
+    constexpr int kBufs = kUp ? 4 : 2;         // staging tiles of a group
+    const int box = kUp ? 0 : quarter >> 1;    // 64-column box of the CTA's columns
+    const int bar_id = 1 + (kUp ? half : half * 2 + box);
+    const bool lead = kUp ? quarter == 0 : (quarter & 1) == 0;  // the warp that stores
+    uint8_t* stg0 = staging + (kUp ? half * 4 : half * 4 + box * 2) * C::kStagingBytes;
     const uint32_t acc_empty_leader0 = map_to_rank(smem_addr(&acc_empty[0]), 0);
     const uint32_t acc_empty_leader1 = map_to_rank(smem_addr(&acc_empty[1]), 0);
-    int lt = 0;
+    int lt = 0, nbuf = 0;
     for (int t = pair; t < ntiles; t += npairs, ++lt) {
       Tile tl;
       const bool tile_ok = decode_tile<false>(p, ix, t, tl);
@@ -1270,7 +1330,8 @@ __global__ void __launch_bounds__(kThreads2, 1)
       int ok = 1;
       if (lane == 0) ok = mbar_wait(&acc_full[ab], acc_phase, abort_flag, kWaitNs) ? 1 : 0;
       ok = __shfl_sync(0xffffffffu, ok, 0);
-      if (!ok) {
+      // one decision for the whole group: its barriers below have no limit
+      if (!group_all(bar_id, kGroup, ok != 0)) {
         if (lane == 0) {
           if (!*abort_flag) set_err(p.err, kErrTimeout);
           *abort_flag = 1;
@@ -1280,75 +1341,76 @@ __global__ void __launch_bounds__(kThreads2, 1)
       tc_fence_after();
       const uint32_t tbase = tmem_base + (static_cast<uint32_t>(quarter * 32) << 16) +
                              static_cast<uint32_t>(ab * BN);
-      // rows of this warp that belong to the tile (0 when the tile is bad)
-      const int nrows = tile_ok ? max(0, min(32, tl.rows - wrow0)) : 0;
-      const int64_t row_base = static_cast<int64_t>(tl.row0) + wrow0;
       const uint32_t release_bar = ab ? acc_empty_leader1 : acc_empty_leader0;
       auto hand_back = [&]() {
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive_cluster_relaxed(release_bar);
       };
-      if (MODE == kModeSwiGLU) {
-        // output columns [64 half, +64): gate at c, up at BN/2 + c; both
-        // 32-column rounds fill one 128-byte staging row
-        staging_free();
+      const int nchunks = tile_ok ? tile_cols(tl.rows) / 32 : 0;
+      // first output column of the group's staging tile
+      const int col0 = kUp ? tl.n * 128 + static_cast<int>(rank) * 64
+                           : tl.n * 256 + static_cast<int>(rank) * BM + box * 64;
+      if (half >= nchunks) hand_back();
+      for (int c = half; c < nchunks; c += 2) {
+        // SwiGLU: gate rows (lanes 0-15) and the matching up rows (16-31) of
+        // the same columns and tokens; down: the first and the last 16 columns
+        uint32_t v0[16], v1[16];
+        tmem_ld_frag(tbase + 32 * c, v0);
+        tmem_ld_frag(tbase + (16u << 16) + 32 * c, v1);
+        tmem_ld_wait();
+        if (c + 2 >= nchunks) hand_back();
+        uint8_t* stg = stg0 + (nbuf % kBufs) * C::kStagingBytes;
+        const uint32_t stg_s = smem_addr(stg);
+        // the store that last used this staging tile has read it
+        if (lead && lane == 0) bulk_wait_read<kBufs - 1>();
+        group_sync(bar_id, kGroup);
+        const int mrow = lane & 7, mat = lane >> 3;  // of the row this thread addresses
+        if (kUp) {
+          uint32_t w[8];  // [8-token group][8-column block]
 #pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const int c = half * 64 + 32 * r;
-          uint32_t g[32], u[32];
-          tmem_ld32(tbase + c, g);
-          tmem_ld32(tbase + BN / 2 + c, u);
-          tmem_ld_wait();
-          if (r == 1) hand_back();
-          uint32_t packed[16];
+          for (int i = 0; i < 8; ++i) {
+            float act[2];
 #pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            const float g0 = __uint_as_float(g[2 * i]), g1 = __uint_as_float(g[2 * i + 1]);
-            const float u0 = __uint_as_float(u[2 * i]), u1 = __uint_as_float(u[2 * i + 1]);
-            const float a0 = g0 / (1.0f + __expf(-g0)) * u0;
-            const float a1 = g1 / (1.0f + __expf(-g1)) * u1;
-            __nv_bfloat162 h2 = __floats2bfloat162_rn(a0, a1);
-            packed[i] = *reinterpret_cast<uint32_t*>(&h2);
+            for (int h = 0; h < 2; ++h) {
+              const float gt = __uint_as_float(v0[2 * i + h]), up = __uint_as_float(v1[2 * i + h]);
+              act[h] = gt / (1.0f + __expf(-gt)) * up;
+            }
+            w[i] = pack_bf16(act[0], act[1]);
           }
+          // matrices: token groups 2 m and 2 m + 1, column blocks 0 and 1 of each
 #pragma unroll
-          for (int v = 0; v < 4; ++v)
-            stage_chunk(stg, lane, 4 * r + v,
-                        make_uint4(packed[4 * v], packed[4 * v + 1], packed[4 * v + 2],
-                                   packed[4 * v + 3]));
+          for (int m = 0; m < 2; ++m)
+            stmatrix_trans(stage_addr(stg_s, 8 * (2 * m + (mat >> 1)) + mrow,
+                                      quarter * 2 + (mat & 1)),
+                           w[4 * m], w[4 * m + 1], w[4 * m + 2], w[4 * m + 3]);
+        } else {
+          // one token group per store, its four column blocks
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            stmatrix_trans(stage_addr(stg_s, 8 * j + mrow, (quarter & 1) * 4 + mat),
+                           pack_bf16(v0[4 * j], v0[4 * j + 1]),
+                           pack_bf16(v0[4 * j + 2], v0[4 * j + 3]),
+                           pack_bf16(v1[4 * j], v1[4 * j + 1]),
+                           pack_bf16(v1[4 * j + 2], v1[4 * j + 3]));
         }
-        emit(row_base, tl.n * (BN / 2) + half * 64, nrows);
-      } else {
-        // columns [128 half, +128) in two rounds of 64 (one staging row each)
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          const int c = half * 128 + 64 * r;
-          uint32_t v0[32], v1[32];
-          tmem_ld32(tbase + c, v0);
-          tmem_ld32(tbase + c + 32, v1);
-          tmem_ld_wait();
-          if (r == 1) hand_back();
-          uint32_t packed[32];
-#pragma unroll
-          for (int i = 0; i < 16; ++i) {
-            __nv_bfloat162 h0 = __floats2bfloat162_rn(__uint_as_float(v0[2 * i]),
-                                                      __uint_as_float(v0[2 * i + 1]));
-            __nv_bfloat162 h1 = __floats2bfloat162_rn(__uint_as_float(v1[2 * i]),
-                                                      __uint_as_float(v1[2 * i + 1]));
-            packed[i] = *reinterpret_cast<uint32_t*>(&h0);
-            packed[16 + i] = *reinterpret_cast<uint32_t*>(&h1);
+        fence_proxy_async_smem();  // the staging writes, before the store reads them
+        group_sync(bar_id, kGroup);
+        if (lead) {
+          const int nrows = min(32, tl.rows - 32 * c);
+          if (nrows == 32) {
+            if (lane == 0)
+              tma_store_2d(&map_out, smem_addr(stg), col0, tl.row0 + 32 * c);
+          } else {
+            flush_staging(stg, lane, p.out, static_cast<int64_t>(tl.row0) + 32 * c, p.ldo, col0,
+                          nrows);
           }
-          staging_free();
-#pragma unroll
-          for (int v = 0; v < 8; ++v)
-            stage_chunk(stg, lane, v,
-                        make_uint4(packed[4 * v], packed[4 * v + 1], packed[4 * v + 2],
-                                   packed[4 * v + 3]));
-          emit(row_base, tl.n * BN + c, nrows);
+          if (lane == 0) bulk_commit();  // a group per chunk, empty for lane stores
         }
+        ++nbuf;
       }
     }
-    if (tma_out && lane == 0) bulk_wait_all();  // every store written before exit
+    if (lead && lane == 0) bulk_wait_all();  // every store written before exit
   }
 
   tc_fence_before();
@@ -1369,9 +1431,10 @@ cudaError_t launch_pair_impl(const TcGemmArgs& a, cudaStream_t stream) {
                                        C::kSmemBytes);
   if (e != cudaSuccess) return e;
   if (a.K % (BK * C::KS) != 0) return cudaErrorInvalidValue;  // whole stages
+  if (a.map_x == nullptr || a.map_out == nullptr) return cudaErrorInvalidValue;
   KParams p;
   p.K = a.K;
-  p.n_tiles = MODE == kModeSwiGLU ? a.n_total / (C::BN / 2) : a.n_total / C::BN;
+  p.n_tiles = MODE == kModeSwiGLU ? a.n_total / 128 : a.n_total / 256;
   p.b_rows_per_group = a.b_rows_per_group;
   p.b_up_offset = a.b_up_offset;
   p.g = a.g;
@@ -1391,7 +1454,6 @@ cudaError_t launch_pair_impl(const TcGemmArgs& a, cudaStream_t stream) {
   p.early_b = a.early_b ? 1 : 0;
   p.b3d = 0;
   p.norm_out = nullptr;
-  p.tma_out = a.map_out != nullptr ? 1 : 0;
   p.gather_perm = MODE == kModeSwiGLU ? a.gather_perm : nullptr;
   p.gather_kmax = a.gather_kmax;
   p.gather_tokens = a.gather_tokens;
@@ -1416,9 +1478,8 @@ cudaError_t launch_pair_impl(const TcGemmArgs& a, cudaStream_t stream) {
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  // without an output map the per-lane stores run and map_a stands in
-  return cudaLaunchKernelEx(&cfg, kernel, *a.map_a, *a.map_b,
-                            a.map_out != nullptr ? *a.map_out : *a.map_a, p);
+  return cudaLaunchKernelEx(&cfg, kernel, *a.map_b, a.map_x[0], a.map_x[1], a.map_x[2],
+                            a.map_x[3], *a.map_out, p);
 }
 
 }  // namespace

@@ -199,7 +199,7 @@ struct TcGemmArgs {
   // SwiGLU, 1-SM kernel: map_b is the 3D map of tc_gate_up_3d (box {64,
   // bn / 2, 2}: a tile's gate and up rows in one copy) instead of a 2D map
   bool b_gate_up_3d = false;
-  // SwiGLU, CTA-pair kernel: when set, map_a is a {64, 1}-box map of the
+  // SwiGLU, CTA-pair kernel: when set, map_x[0] is a {64, 1}-box map of the
   // token rows X [gather_tokens, K], and A row r is token gather_perm[r] /
   // gather_kmax (row r's pair index over k_max), fetched by four-row TMA
   // gathers; nullptr: map_a holds the rows in pair order
@@ -208,8 +208,11 @@ struct TcGemmArgs {
   int gather_tokens = 0;
   // CTA-pair kernels: 2D map of out [rows, ldo] with a {64, 32} box, 128-byte
   // swizzle; whole 32-row output chunks are written by TMA stores through it
-  // (nullptr: per-lane stores)
   const CUtensorMap* map_out = nullptr;
+  // CTA-pair kernels (instead of map_a): four maps of A with boxes of 32, 64,
+  // 96 and 128 rows; with gather_perm the first is the {64, 1}-box map of the
+  // token rows
+  const CUtensorMap* map_x = nullptr;
   // 1-SM kernels, grouped rows: a dense problem (the shared expert) whose
   // tiles the same launch computes; map_b of the kind of this one, n_total a
   // multiple of the tile's columns
@@ -236,9 +239,11 @@ int tc_b_box_rows(bool swiglu, int bn);
 cudaError_t launch_scores_tc(const TcGemmArgs& a, int bn, int k_splits, float* out,
                              int64_t split_stride, int n_valid, bool defer_wait,
                              cudaStream_t stream, float* row_norms = nullptr);
-// CTA-pair (2-SM, cta_group::2) variants: 256 x 256 tiles, cluster of two
-// CTAs; A and B tensor maps both with boxes of 128 rows; needs
-// GroupRows::mt2_prefix in grouped mode.  n_total must be a multiple of 128
+// CTA-pair (2-SM, cta_group::2) variants: tiles of 256 weight rows x up to
+// 256 token rows, cluster of two CTAs; needs map_x, map_out and
+// GroupRows::mt2_prefix in grouped mode.  map_b: SwiGLU a 5D map {K, 16, 2,
+// inter / 16, groups} of the gate/up weights with box {64, 16, 2, 4, 1}, down
+// a 2D map with boxes of 128 rows.  n_total must be a multiple of 128
 // (SwiGLU) or 256 (down).
 cudaError_t launch_swiglu_tc_pair(const TcGemmArgs& a, cudaStream_t stream);
 cudaError_t launch_down_tc_pair(const TcGemmArgs& a, cudaStream_t stream);

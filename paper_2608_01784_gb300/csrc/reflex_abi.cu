@@ -157,6 +157,35 @@ bool make_map_gate_up(CUtensorMap* m, const void* base, int64_t groups, int64_t 
   return r == CUDA_SUCCESS;
 }
 
+// The same weights for the CTA-pair kernel, as {K, 16, 2, inter / 16, groups}:
+// one box {64, 16, 2, 4, 1} holds 64 gate and the matching 64 up rows, 16 of
+// each in turn.
+bool make_map_gate_up_pair(CUtensorMap* m, const void* base, int64_t groups, int64_t inter,
+                           int64_t cols) {
+  auto fn = encode_fn();
+  if (fn == nullptr) return false;
+  if ((reinterpret_cast<uintptr_t>(base) & 15) != 0) return false;
+  const cuuint64_t row = static_cast<cuuint64_t>(cols) * 2;
+  cuuint64_t dims[5] = {static_cast<cuuint64_t>(cols), 16, 2,
+                        static_cast<cuuint64_t>(inter / 16), static_cast<cuuint64_t>(groups)};
+  cuuint64_t strides[4] = {row, row * static_cast<cuuint64_t>(inter), row * 16,
+                           row * 2 * static_cast<cuuint64_t>(inter)};
+  cuuint32_t box[5] = {64, 16, 2, 4, 1};
+  cuuint32_t estr[5] = {1, 1, 1, 1, 1};
+  CUresult r = fn(m, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 5, const_cast<void*>(base),
+                  dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
+                  CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                  CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+  return r == CUDA_SUCCESS;
+}
+
+// Token-row maps of the CTA-pair kernel: boxes of 32, 64, 96 and 128 rows.
+bool make_maps_x(CUtensorMap* m, const void* base, int64_t rows, int64_t cols) {
+  for (int i = 0; i < 4; ++i)
+    if (!make_map(m + i, base, rows, cols, 32 * (i + 1))) return false;
+  return true;
+}
+
 int map_err_bits(uint32_t bits) {
   if (bits == 0) return REFLEX_OK;
   if (bits & rx::kErrTimeout) return REFLEX_ETIMEOUT;
@@ -565,15 +594,22 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
       }
     } else {
       CUtensorMap ma1, mb1, ma2, mb2;
-      if (!(gemm_gathers ? make_map(&ma1, hidden, T, d, 1)
-                         : make_map(&ma1, xperm, cap, d, rx::kTileM)) ||
-          !(pair_routed ? make_map(&mb1, w_gate_up, static_cast<int64_t>(E) * 2 * inter, d, 128)
-                        : make_map_gate_up(&mb1, w_gate_up, E, inter, d,
-                                           rx::tc_b_box_rows(true, bn_up))) ||
-          !make_map(&ma2, amid, cap, inter, rx::kTileM) ||
-          !make_map(&mb2, w_down, static_cast<int64_t>(E) * d, inter,
-                    pair_routed ? 128 : rx::tc_b_box_rows(false, bn_dn)))
+      CUtensorMap x1[4], x2[4], mo1, mo2;  // CTA pairs: rows by box height, outputs
+      if (pair_routed) {
+        if (!make_maps_x(x1, xperm, cap, d) || !make_maps_x(x2, amid, cap, inter) ||
+            (gemm_gathers && !make_map(x1, hidden, T, d, 1)) ||
+            !make_map_gate_up_pair(&mb1, w_gate_up, E, inter, d) ||
+            !make_map(&mb2, w_down, static_cast<int64_t>(E) * d, inter, 128) ||
+            !make_map(&mo1, amid, cap, inter, 32) || !make_map(&mo2, xperm, cap, d, 32))
+          return REFLEX_ECUDA;
+      } else if (!make_map(&ma1, xperm, cap, d, rx::kTileM) ||
+                 !make_map_gate_up(&mb1, w_gate_up, E, inter, d,
+                                   rx::tc_b_box_rows(true, bn_up)) ||
+                 !make_map(&ma2, amid, cap, inter, rx::kTileM) ||
+                 !make_map(&mb2, w_down, static_cast<int64_t>(E) * d, inter,
+                           rx::tc_b_box_rows(false, bn_dn))) {
         return REFLEX_ECUDA;
+      }
       rx::TcGemmArgs g1{&ma1, &mb1, d, inter, 2 * inter, inter, grouped, amid, inter, err, sms,
                         !pair_routed};
       if (gemm_gathers) {
@@ -582,11 +618,9 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
         g1.gather_tokens = T;
       }
       rx::TcGemmArgs g2{&ma2, &mb2, inter, d, d, 0, grouped, xperm, d, err, sms};
-      // output maps of the CTA-pair GEMMs (whole 32-row chunks by TMA store)
-      CUtensorMap mo1, mo2;
       if (pair_routed) {
-        if (!make_map(&mo1, amid, cap, inter, 32) || !make_map(&mo2, xperm, cap, d, 32))
-          return REFLEX_ECUDA;
+        g1.map_x = x1;
+        g2.map_x = x2;
         g1.map_out = &mo1;
         g2.map_out = &mo2;
       }
@@ -605,24 +639,28 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
       const bool pair_shared = shared_inter > 0 && !carry_shared && T >= 2048 &&
                                shared_inter % 128 == 0 && d % 256 == 0;
       const int bn_s1 = carry_shared ? bn_up : bn_sup, bn_s2 = carry_shared ? bn_dn : bn_sdn;
-      CUtensorMap sa1, sb1, sa2, sb2;
-      if (shared_inter &&
-          (!make_map(&sa1, hidden, T, d, rx::kTileM) ||
-           !(pair_shared
-                 ? make_map(&sb1, shared_gate_up, 2 * static_cast<int64_t>(shared_inter), d, 128)
-                 : make_map_gate_up(&sb1, shared_gate_up, 1, shared_inter, d,
-                                    rx::tc_b_box_rows(true, bn_s1))) ||
-           !make_map(&sa2, ash, T, shared_inter, rx::kTileM) ||
-           !make_map(&sb2, shared_down, d, shared_inter,
-                     pair_shared ? 128 : rx::tc_b_box_rows(false, bn_s2))))
+      CUtensorMap sa1, sb1, sa2, sb2, sx1[4], sx2[4], so1, so2;
+      if (pair_shared) {
+        if (!make_maps_x(sx1, hidden, T, d) || !make_maps_x(sx2, ash, T, shared_inter) ||
+            !make_map_gate_up_pair(&sb1, shared_gate_up, 1, shared_inter, d) ||
+            !make_map(&sb2, shared_down, d, shared_inter, 128) ||
+            !make_map(&so1, ash, T, shared_inter, 32) || !make_map(&so2, ysh, T, d, 32))
+          return REFLEX_ECUDA;
+      } else if (shared_inter &&
+                 (!make_map(&sa1, hidden, T, d, rx::kTileM) ||
+                  !make_map_gate_up(&sb1, shared_gate_up, 1, shared_inter, d,
+                                    rx::tc_b_box_rows(true, bn_s1)) ||
+                  !make_map(&sa2, ash, T, shared_inter, rx::kTileM) ||
+                  !make_map(&sb2, shared_down, d, shared_inter,
+                            rx::tc_b_box_rows(false, bn_s2)))) {
         return REFLEX_ECUDA;
+      }
       rx::TcGemmArgs h1{&sa1, &sb1, d, shared_inter, 2 * shared_inter, shared_inter,
                         dense, ash, shared_inter, err, sms, !pair_shared};
       rx::TcGemmArgs h2{&sa2, &sb2, shared_inter, d, d, 0, dense, ysh, d, err, sms};
-      CUtensorMap so1, so2;
       if (pair_shared) {
-        if (!make_map(&so1, ash, T, shared_inter, 32) || !make_map(&so2, ysh, T, d, 32))
-          return REFLEX_ECUDA;
+        h1.map_x = sx1;
+        h2.map_x = sx2;
         h1.map_out = &so1;
         h2.map_out = &so2;
       }
