@@ -73,14 +73,14 @@ extern "C" {
 #define REFLEX_FLAG_EXACT_SCORES 0x8u
 /* bf16 tcgen05 path, routed gate/up GEMM on CTA pairs (at least 128 rows
  * per expert expected: T * k_max / (2 E) >= 128, inter % 128 == 0, d % 256
- * == 0): the GEMM fetches its input rows from hidden itself with four-row
- * TMA gathers through the pair permutation, and DISPATCH only places the
- * pairs (no copy of the rows in pair order is written).  The outputs are the
- * same bits as without the flag.  Elsewhere the flag changes nothing.  The
- * fused dispatch is slower on GB300 (a four-row gather costs about four
- * times what a row of a tiled box does: the 32 x 1024-token LLaDA-MoE layer's
- * gate/up GEMM 0.84 -> 3.08 ms), so it is off by default.  With stage
- * selection the DISPATCH and EXPERT_UP calls must agree on the flag. */
+ * == 0): the GEMM fetches its input rows from hidden itself through the pair
+ * permutation, and DISPATCH only places the pairs (no copy of the rows in
+ * pair order is written).  The outputs are the same bits as without the flag.
+ * Elsewhere the flag changes nothing.  The fused dispatch is slower on GB300
+ * (row copies by the GEMM's own warps do not keep up with the tensor cores:
+ * the 32 x 1024-token LLaDA-MoE layer's gate/up GEMM 0.78 -> about 1.5 ms),
+ * so it is off by default.  With stage selection the DISPATCH and EXPERT_UP
+ * calls must agree on the flag. */
 #define REFLEX_FLAG_GATHER_IN_GEMM 0x10u
 /* Stage selection.  No stage bit = all five stages in order.  Stages read
  * what the previous stages left in the same workspace; running a stage whose

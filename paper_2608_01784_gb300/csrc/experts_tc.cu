@@ -107,6 +107,7 @@ struct KParams {
   int early_b;
   // SwiGLU on CTA pairs: A rows gathered from the token rows (TcGemmArgs)
   const int32_t* gather_perm;
+  const __nv_bfloat16* gather_x;
   int gather_kmax;
   int gather_tokens;
 };
@@ -794,6 +795,7 @@ cudaError_t launch_impl(const TcGemmArgs& a, cudaStream_t stream) {
   p.b3d = MODE == kModeSwiGLU && a.b_gate_up_3d ? 1 : 0;
   p.norm_out = nullptr;
   p.gather_perm = nullptr;
+  p.gather_x = nullptr;
   p.gather_kmax = 1;
   p.gather_tokens = 0;
   set_shared_problem(p, SH ? a.shared : nullptr, MODE == kModeSwiGLU ? BN / 2 : BN);
@@ -821,11 +823,12 @@ cudaError_t launch_impl(const TcGemmArgs& a, cudaStream_t stream) {
 // meet in one warp's TMEM lanes, 16 apart.  Down: rows n*256 + 128 r of
 // W_down.  A 192 KB ring holds 3 stages of two consecutive 64-k blocks, at
 // most 32 KB per SM and block.  With gathered rows (SwiGLU,
-// TcGemmArgs::gather_perm) the rows come straight from the token rows: every
-// lane of the producer warp issues one four-row TMA gather per 64-k block,
-// the tokens looked up through the pair permutation once per tile; the rows,
-// tiles and MMA order are those of the copied rows, so the outputs are the
-// same bits.  One thread of the leader CTA (rank 0) issues
+// TcGemmArgs::gather_perm) four more warps copy the rows straight from the
+// token rows (cp.async, the tokens looked up through the pair permutation);
+// the rows, tiles and MMA order are those of the copied rows, so the outputs
+// are the same bits.  Their two stages in flight do not cover the L2 latency
+// (32768 tokens x 64 experts: gate/up 0.78 -> 1.53 ms), so it is opt-in;
+// four-row TMA gathers before them took 3.08 ms.  One thread of the leader CTA (rank 0) issues
 // tcgen05.mma.cta_group::2; each CTA's TMEM receives its 128 weight rows x
 // the tile's token columns (two buffers of 256 columns, allocated
 // collectively by one warp per CTA).
@@ -839,6 +842,9 @@ cudaError_t launch_impl(const TcGemmArgs& a, cudaStream_t stream) {
 // TMEM lane quarter, each draining half of the accumulator's columns)
 constexpr int kThreads2 = 320;
 constexpr int kEpiWarps2 = 8;
+// SwiGLU: four more warps (10-13) that gather the token rows
+constexpr int kGatherWarps = 4;
+constexpr int kThreads2Up = kThreads2 + 32 * kGatherWarps;
 
 __device__ __forceinline__ uint32_t cluster_rank() {
   uint32_t r;
@@ -892,18 +898,43 @@ __device__ __forceinline__ void tma_load_5d_pair(uint32_t dst, const CUtensorMap
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(0), "r"(c3), "r"(c4), "r"(cl_bar)
       : "memory");
 }
-// Four rows r0..r3 of a map whose box is {64, 1}, copied to four consecutive
-// 128-byte rows at dst (the same 128-byte swizzle as a tiled box: it follows
-// the shared-memory address, and dst is 512-byte aligned, half of an 8-row
-// swizzle atom), completion counted on a barrier in either CTA of the pair.
-__device__ __forceinline__ void tma_gather4_pair(uint32_t dst, const CUtensorMap* map, int c0,
-                                                 const int (&r)[4], uint32_t cl_bar) {
-  asm volatile(
-      "cp.async.bulk.tensor.2d.shared::cluster.global.tile::gather4.mbarrier::complete_tx::bytes"
-      ".cta_group::2 [%0], [%1, {%2, %3, %4, %5, %6}], [%7];" ::"r"(dst),
-      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]),
-      "r"(cl_bar)
-      : "memory");
+// 16 bytes of a gathered row into shared memory, and the hand-over of a stage
+// whose rows came that way: the copies have landed (wait_group), are visible
+// to the tensor core's reads (proxy fence), and count as one arrival on the
+// leader's barrier.
+__device__ __forceinline__ void cp_async_row(uint32_t dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_commit_group() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int N>
+__device__ __forceinline__ void cp_async_wait_but() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+// mbar_wait that also acquires what the other CTA's warps released
+__device__ __forceinline__ bool mbar_wait_cluster(uint64_t* bar, uint32_t parity,
+                                                  const volatile int* abort, uint64_t limit_ns) {
+  uint64_t t0 = 0;
+  for (;;) {
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t"
+        "mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}\n"
+        : "=r"(ok)
+        : "r"(smem_addr(bar)), "r"(parity)
+        : "memory");
+    if (ok) return true;
+    if (abort != nullptr && *abort) return false;
+    const uint64_t now = global_ns();
+    if (t0 == 0) t0 = now;
+    if (now - t0 > limit_ns) return false;
+  }
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cl_bar) {
+  asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];" ::"r"(cl_bar)
+               : "memory");
 }
 __device__ __forceinline__ void mma_bf16_pair(uint32_t tmem_d, uint64_t da, uint64_t db,
                                               uint32_t idesc, uint32_t accumulate) {
@@ -1048,7 +1079,7 @@ __device__ __forceinline__ void flush_staging(const uint8_t* stg, int lane,
 __device__ __forceinline__ int tile_cols(int rows) { return (rows + 31) & ~31; }
 
 template <int MODE>
-__global__ void __launch_bounds__(kThreads2, 1)
+__global__ void __launch_bounds__(MODE == kModeSwiGLU ? kThreads2Up : kThreads2, 1)
     grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w,
                              const __grid_constant__ CUtensorMap map_x32,
                              const __grid_constant__ CUtensorMap map_x64,
@@ -1082,9 +1113,11 @@ __global__ void __launch_bounds__(kThreads2, 1)
   const int pair = blockIdx.x >> 1;
   const int npairs = gridDim.x >> 1;
 
+  const bool gather = MODE == kModeSwiGLU && p.gather_perm != nullptr;
   if (threadIdx.x == 0) {
     for (int s = 0; s < kStages; ++s) {
-      mbar_init(&full[s], 2);  // one expect_tx arrival per CTA of the pair
+      // one expect_tx arrival per CTA of the pair (+ one per gather warp)
+      mbar_init(&full[s], gather ? 2 + 2 * kGatherWarps : 2);
       mbar_init(&empty[s], 1);
     }
     for (int b = 0; b < 2; ++b) {
@@ -1111,7 +1144,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
   // the ring's first weights while the kernel in front still runs, as in the
   // 1-SM kernel; both CTAs' bytes count on the leader's barriers
   int early = 0;  // stages whose weights are on their way (warp 0)
-  if (p.early_b && p.gather_perm == nullptr && warp == 0) {
+  if (p.early_b && warp == 0) {
     Tile tl;
     if (early_tile<false>(p, pair, tl)) {
       early = nk < kStages ? nk : kStages;
@@ -1141,11 +1174,7 @@ __global__ void __launch_bounds__(kThreads2, 1)
   // counts 256-row tiles
   const int ntiles = total_tiles<false>(p, ix);
 
-  // SwiGLU with gathered rows: the whole producer warp issues the row copies,
-  // one four-row gather per lane and 64-k block (lane l: rows 4 l .. 4 l + 3
-  // of this CTA's half); otherwise lane 0 issues everything
-  const bool gather = MODE == kModeSwiGLU && p.gather_perm != nullptr;
-  if (warp == 0 && (gather || lane == 0)) {
+  if (warp == 0 && lane == 0) {
     // ---------------- TMA producer (each CTA: its weight rows, its token rows)
     int stage = 0;
     uint32_t phase = 0;
@@ -1153,11 +1182,9 @@ __global__ void __launch_bounds__(kThreads2, 1)
     bool ok = true;
     for (int t = pair; t < ntiles && ok; t += npairs) {
       Tile tl;
-      if (!decode_tile<false>(p, ix, t, tl)) {  // the same outcome in every lane
-        if (lane == 0) {
-          set_err(p.err, kErrIndex);
-          *abort_flag = 1;
-        }
+      if (!decode_tile<false>(p, ix, t, tl)) {
+        set_err(p.err, kErrIndex);
+        *abort_flag = 1;
         break;
       }
       const int half_rows = tile_cols(tl.rows) / 2;  // token rows per CTA, a multiple of 16
@@ -1167,57 +1194,29 @@ __global__ void __launch_bounds__(kThreads2, 1)
       const int bx = (half_rows + 31) / 32;
       const CUtensorMap* mx = bx == 1 ? &map_x32 : bx == 2 ? &map_x64 : bx == 3 ? &map_x96
                                                                              : &map_x128;
-      const uint32_t xbytes = gather ? C::kXBytes : static_cast<uint32_t>(C::KS * bx * 32 * 128);
-      // token of each of this lane's four rows; rows past the tile's end
-      // repeat its last row (computed, never stored)
-      int tok[4] = {0, 0, 0, 0};
-      if (gather) {
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-          const int r = min(static_cast<int>(rank) * half_rows + min(4 * lane + i, half_rows - 1),
-                            tl.rows - 1);
-          const int o = p.gather_perm[tl.row0 + r];
-          const int tk = o >= 0 ? o / p.gather_kmax : -1;
-          if (tk < 0 || tk >= p.gather_tokens)
-            set_err(p.err, kErrIndex);
-          else
-            tok[i] = tk;
-        }
-      }
+      const uint32_t xbytes = gather ? 0u : static_cast<uint32_t>(C::KS * bx * 32 * 128);
       for (int kb = 0; kb < nk; ++kb) {
-        // every issuing lane observes the stage's release itself
-        const bool w = mbar_wait(&empty[stage], phase ^ 1u, abort_flag, kWaitNs);
-        if (!(gather ? __all_sync(0xffffffffu, w) : w)) {
+        if (!mbar_wait(&empty[stage], phase ^ 1u, abort_flag, kWaitNs)) {
           ok = false;
           break;
         }
         const uint32_t fb = map_to_rank(smem_addr(&full[stage]), 0);
         const bool ahead = early > 0;  // the weights are already on their way
         if (ahead) --early;
-        if (lane == 0) {
-          const uint32_t bytes = (ahead ? 0u : static_cast<uint32_t>(C::kWBytes)) + xbytes;
-          if (leader)
-            mbar_expect_tx(smem_addr(&full[stage]), bytes);
-          else
-            mbar_expect_tx_cluster(fb, bytes);
-          // consecutive k blocks of the same rows back to back
+        const uint32_t bytes = (ahead ? 0u : static_cast<uint32_t>(C::kWBytes)) + xbytes;
+        if (leader)
+          mbar_expect_tx(smem_addr(&full[stage]), bytes);
+        else
+          mbar_expect_tx_cluster(fb, bytes);
+        // consecutive k blocks of the same rows back to back
 #pragma unroll
-          for (int u = 0; u < C::KS; ++u) {
-            const int k0 = (kb * C::KS + u) * BK;
-            if (!gather)
-              tma_load_2d_pair(smem_addr(sx + stage * C::kXBytes + u * C::kSubBytes), mx, k0,
-                               xrow, fb);
-            if (!ahead)
-              load_weights(tl, smem_addr(sw + stage * C::kWBytes + u * C::kSubBytes), k0, fb);
-          }
-        }
-        if (gather) {
-          __syncwarp();
-#pragma unroll
-          for (int u = 0; u < C::KS; ++u)
-            tma_gather4_pair(
-                smem_addr(sx + stage * C::kXBytes + u * C::kSubBytes + lane * 4 * 128), &map_x32,
-                (kb * C::KS + u) * BK, tok, fb);
+        for (int u = 0; u < C::KS; ++u) {
+          const int k0 = (kb * C::KS + u) * BK;
+          if (!gather)
+            tma_load_2d_pair(smem_addr(sx + stage * C::kXBytes + u * C::kSubBytes), mx, k0, xrow,
+                             fb);
+          if (!ahead)
+            load_weights(tl, smem_addr(sw + stage * C::kWBytes + u * C::kSubBytes), k0, fb);
         }
         issued_mask |= 1u << stage;
         issued_phase = (issued_phase & ~(1u << stage)) | (phase << stage);
@@ -1227,27 +1226,24 @@ __global__ void __launch_bounds__(kThreads2, 1)
         }
       }
     }
-    if (lane == 0) {
-      if (!ok) {
-        set_err(p.err, kErrTimeout);
-        *abort_flag = 1;
+    if (!ok) {
+      set_err(p.err, kErrTimeout);
+      *abort_flag = 1;
+    }
+    // early weights of stages that never got their rows: the arrivals that
+    // are missing come from both CTAs, and the leader sees the bytes land
+    for (int s = 0; s < early; ++s) {
+      const int st = (stage + s) % kStages;
+      for (int n = 0; n < (gather ? 1 + kGatherWarps : 1); ++n) {
+        if (leader) mbar_arrive1(smem_addr(&full[st]));
+        else mbar_arrive_cluster_relaxed(map_to_rank(smem_addr(&full[st]), 0));
       }
-      // early weights of stages that never got their rows: both CTAs arrive,
-      // and the leader sees the bytes of both land
-      for (int s = 0; s < early; ++s) {
-        const int st = (stage + s) % kStages;
-        if (leader) {
-          mbar_arrive1(smem_addr(&full[st]));
-          mbar_wait(&full[st], 0, nullptr, kDrainNs);
-        } else {
-          mbar_arrive_cluster_relaxed(map_to_rank(smem_addr(&full[st]), 0));
-        }
-      }
-      if (*abort_flag && leader) {
-        for (int s = 0; s < kStages; ++s)
-          if (issued_mask & (1u << s))
-            mbar_wait(&full[s], (issued_phase >> s) & 1u, nullptr, kDrainNs);
-      }
+      if (leader) mbar_wait(&full[st], 0, nullptr, kDrainNs);
+    }
+    if (*abort_flag && leader) {
+      for (int s = 0; s < kStages; ++s)
+        if (issued_mask & (1u << s))
+          mbar_wait(&full[s], (issued_phase >> s) & 1u, nullptr, kDrainNs);
     }
   } else if (warp == 1 && lane == 0 && leader) {
     // ---------------- MMA issuer (leader CTA only) ----------------
@@ -1270,7 +1266,8 @@ __global__ void __launch_bounds__(kThreads2, 1)
       tc_fence_after();
       const uint32_t d_tmem = tmem_base + static_cast<uint32_t>(ab * BN);
       for (int kb = 0; kb < nk; ++kb) {
-        if (!mbar_wait(&full[stage], phase, abort_flag, kWaitNs)) {
+        if (!(gather ? mbar_wait_cluster(&full[stage], phase, abort_flag, kWaitNs)
+                     : mbar_wait(&full[stage], phase, abort_flag, kWaitNs))) {
           ok = false;
           break;
         }
@@ -1301,6 +1298,84 @@ __global__ void __launch_bounds__(kThreads2, 1)
     if (*abort_flag && issued_any) {
       mma_commit_pair(smem_addr(drain));
       mbar_wait(drain, 0, nullptr, kDrainNs);
+    }
+  } else if (MODE == kModeSwiGLU && warp >= 2 + kEpiWarps2) {
+    // ---------------- row gather (each CTA: its half of the tile's rows) -------
+    // Warp g copies rows 32 g .. +31 of the half, eight lanes per row segment
+    // of 128 bytes, into the swizzled stage; lane l handles rows 4 i + l / 8.
+    // A stage is handed over once the next one's copies are on their way, so
+    // two stages are in flight; the next tile's rows are looked up a tile
+    // ahead.
+    if (gather) {
+      const int g0 = (warp - 2 - kEpiWarps2) * 32 + (lane >> 3);
+      const int ch = lane & 7;
+      int tok[8], next[8], half_rows = 0, next_half = 0;
+      auto look_up = [&](int t, int (&tk)[8], int& hr) {
+        Tile tl;
+        hr = 0;
+        if (t >= ntiles || !decode_tile<false>(p, ix, t, tl)) return;
+        hr = tile_cols(tl.rows) / 2;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          // rows past the tile's end repeat its last row (never stored)
+          const int r = min(static_cast<int>(rank) * hr + min(g0 + 4 * i, hr - 1), tl.rows - 1);
+          tk[i] = p.gather_perm[tl.row0 + r];
+        }
+      };
+      int stage = 0, prev = -1;
+      uint32_t phase = 0;
+      bool ok = true;
+      auto hand_over = [&](int st) {
+        fence_proxy_async_smem();  // this lane's landed copies, before the MMAs read them
+        __syncwarp();
+        if (lane == 0) mbar_arrive_cluster(map_to_rank(smem_addr(&full[st]), 0));
+      };
+      look_up(pair, next, next_half);
+      for (int t = pair; t < ntiles && ok; t += npairs) {
+        half_rows = next_half;
+        const __nv_bfloat16* src[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          tok[i] = next[i] >= 0 ? next[i] / p.gather_kmax : -1;
+          if (half_rows > 0 && (tok[i] < 0 || tok[i] >= p.gather_tokens)) {
+            set_err(p.err, kErrIndex);
+            tok[i] = 0;
+          }
+          src[i] = p.gather_x + static_cast<int64_t>(half_rows > 0 ? tok[i] : 0) * p.K + ch * 8;
+        }
+        look_up(t + npairs, next, next_half);
+        if (half_rows == 0) break;  // inconsistent workspace: the producer aborts
+        for (int kb = 0; kb < nk; ++kb) {
+          if (!__all_sync(0xffffffffu,
+                          mbar_wait(&empty[stage], phase ^ 1u, abort_flag, kWaitNs))) {
+            ok = false;
+            break;
+          }
+#pragma unroll
+          for (int u = 0; u < C::KS; ++u) {
+            const uint32_t dst = smem_addr(sx + stage * C::kXBytes + u * C::kSubBytes);
+            const int k0 = (kb * C::KS + u) * BK;
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+              const int r = g0 + 4 * i;
+              if (r < half_rows)
+                cp_async_row(dst + r * 128 + ((ch ^ (r & 7)) << 4), src[i] + k0);
+            }
+          }
+          cp_async_commit_group();
+          if (prev >= 0) {
+            cp_async_wait_but<1>();
+            hand_over(prev);
+          }
+          prev = stage;
+          if (++stage == kStages) {
+            stage = 0;
+            phase ^= 1u;
+          }
+        }
+      }
+      cp_async_wait_but<0>();  // every copy lands before the CTA exits
+      if (ok && prev >= 0) hand_over(prev);
     }
   } else if (warp >= 2) {
     // ---------------- epilogue (each CTA: its 128 weight rows) ----------------
@@ -1455,9 +1530,10 @@ cudaError_t launch_pair_impl(const TcGemmArgs& a, cudaStream_t stream) {
   p.b3d = 0;
   p.norm_out = nullptr;
   p.gather_perm = MODE == kModeSwiGLU ? a.gather_perm : nullptr;
+  p.gather_x = static_cast<const __nv_bfloat16*>(a.gather_x);
   p.gather_kmax = a.gather_kmax;
   p.gather_tokens = a.gather_tokens;
-  if (p.gather_perm != nullptr && (p.gather_kmax < 1 || p.gather_tokens < 1))
+  if (p.gather_perm != nullptr && (p.gather_x == nullptr || p.gather_kmax < 1 || p.gather_tokens < 1))
     return cudaErrorInvalidValue;
   const int64_t max_tiles = static_cast<int64_t>(p.n_tiles) * p.max_mtiles;
   if (max_tiles == 0) return cudaSuccess;
@@ -1466,7 +1542,7 @@ cudaError_t launch_pair_impl(const TcGemmArgs& a, cudaStream_t stream) {
   if (pairs < 1) pairs = 1;
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(2 * pairs);
-  cfg.blockDim = dim3(kThreads2);
+  cfg.blockDim = dim3(MODE == kModeSwiGLU ? kThreads2Up : kThreads2);
   cfg.dynamicSmemBytes = C::kSmemBytes;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
@@ -1548,6 +1624,9 @@ cudaError_t launch_scores_tc(const TcGemmArgs& a, int bn, int k_splits, float* o
                                   row_norms, stream);
   if (bn == 128)
     return launch_scores_impl<128>(a, k_splits, out, split_stride, n_valid, defer_wait,
+                                   row_norms, stream);
+  if (bn == 256)
+    return launch_scores_impl<256>(a, k_splits, out, split_stride, n_valid, defer_wait,
                                    row_norms, stream);
   return cudaErrorInvalidValue;
 }

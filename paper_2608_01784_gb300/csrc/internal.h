@@ -199,19 +199,19 @@ struct TcGemmArgs {
   // SwiGLU, 1-SM kernel: map_b is the 3D map of tc_gate_up_3d (box {64,
   // bn / 2, 2}: a tile's gate and up rows in one copy) instead of a 2D map
   bool b_gate_up_3d = false;
-  // SwiGLU, CTA-pair kernel: when set, map_x[0] is a {64, 1}-box map of the
-  // token rows X [gather_tokens, K], and A row r is token gather_perm[r] /
-  // gather_kmax (row r's pair index over k_max), fetched by four-row TMA
-  // gathers; nullptr: map_a holds the rows in pair order
+  // SwiGLU, CTA-pair kernel: when set, A row r is row gather_perm[r] /
+  // gather_kmax (row r's pair index over k_max) of the token rows gather_x
+  // [gather_tokens, K], copied by four warps of the kernel; nullptr: map_x
+  // holds the rows in pair order
   const int32_t* gather_perm = nullptr;
+  const void* gather_x = nullptr;
   int gather_kmax = 0;
   int gather_tokens = 0;
   // CTA-pair kernels: 2D map of out [rows, ldo] with a {64, 32} box, 128-byte
   // swizzle; whole 32-row output chunks are written by TMA stores through it
   const CUtensorMap* map_out = nullptr;
   // CTA-pair kernels (instead of map_a): four maps of A with boxes of 32, 64,
-  // 96 and 128 rows; with gather_perm the first is the {64, 1}-box map of the
-  // token rows
+  // 96 and 128 rows
   const CUtensorMap* map_x = nullptr;
   // 1-SM kernels, grouped rows: a dense problem (the shared expert) whose
   // tiles the same launch computes; map_b of the kind of this one, n_total a
@@ -230,7 +230,7 @@ cudaError_t launch_down_tc(const TcGemmArgs& a, int bn, cudaStream_t stream);
 int tc_b_box_rows(bool swiglu, int bn);
 // Router-score screen: out[ks][t][e] = sum over the ks-th of k_splits equal
 // slices of k of A[t, k] B[e, k] (fp32 accumulators, dense rows t < T =
-// a.g.dense_rows, columns e < n_valid, row stride a.ldo), bn in {64, 128}
+// a.g.dense_rows, columns e < n_valid, row stride a.ldo), bn in {64, 128, 256}
 // (B tensor map box of bn rows); a.K / 64 must be a multiple of k_splits.
 // defer_wait: launched right behind a kernel that writes none of its inputs
 // or outputs (it then overlaps that kernel and waits for it before exiting).

@@ -597,7 +597,6 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
       CUtensorMap x1[4], x2[4], mo1, mo2;  // CTA pairs: rows by box height, outputs
       if (pair_routed) {
         if (!make_maps_x(x1, xperm, cap, d) || !make_maps_x(x2, amid, cap, inter) ||
-            (gemm_gathers && !make_map(x1, hidden, T, d, 1)) ||
             !make_map_gate_up_pair(&mb1, w_gate_up, E, inter, d) ||
             !make_map(&mb2, w_down, static_cast<int64_t>(E) * d, inter, 128) ||
             !make_map(&mo1, amid, cap, inter, 32) || !make_map(&mo2, xperm, cap, d, 32))
@@ -614,6 +613,7 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
                         !pair_routed};
       if (gemm_gathers) {
         g1.gather_perm = I32(L.perm);
+        g1.gather_x = hidden;
         g1.gather_kmax = k_max;
         g1.gather_tokens = T;
       }
