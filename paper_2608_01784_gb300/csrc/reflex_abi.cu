@@ -494,7 +494,9 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
                             static_cast<int64_t>(T) * E >= batch_screen_min_scores(E);
   if ((stages & REFLEX_STAGE_ROUTE) && batch_screen) {
     CUtensorMap mh, mw, mhb, mwb;
-    const int sbn = E <= 64 ? 64 : 128;  // score tile width
+    // score tile width: 256 reads each token row once for all experts, once
+    // its 128-row tiles alone fill the SMs (65536 tokens: 105 -> 78 us)
+    const int sbn = E <= 64 ? 64 : E <= 128 || T < 128 * sms_h ? 128 : 256;
     if (!make_map(&mh, hidden, T, d, rx::kTileM) || !make_map(&mw, w_router, E, d, sbn) ||
         !make_map(&mhb, hidden, T, d, rx::screen_batch_token_rows(E),
                   CU_TENSOR_MAP_SWIZZLE_NONE) ||
