@@ -80,7 +80,7 @@ def update_state(state: dict, conf_new: torch.Tensor, num_blocks: torch.Tensor,
 
 def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
                   flags: int = B.REFLEX_FLAG_RENORM_TOPK, count_rule: int = 0,
-                  k_max: int = 12) -> int:
+                  k_max: int = 12, inter: int = 512) -> int:
     """Kernels one reflex_step call launches on the tcgen05 path, following the
     library's choices: the count kernel; the score kernel and the selection,
     or (bf16, renormalised weights, >= 128 experts, T E >= 2048 x 256,
@@ -102,7 +102,10 @@ def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
         16384 * 32 if E <= 32 else 4608 * 64 if E <= 64 else 768 * 256)
     n += 3 if (screen or batch_screen) else 2
     n += 1 if T <= 4096 and (T + 31) // 32 * E * 4 <= 160 * 1024 else 2
-    n += 1 + 2 + (2 if shared_inter and T * k_max // 2 // E >= 128 else 0) + 1
+    est = T * k_max // 2 // E
+    pairs = est >= 128 or (est >= 96 and T >= 2048 and
+                           T * k_max // 2 * (2 * d + inter) * 2 <= 128 << 20)
+    n += 1 + 2 + (2 if shared_inter and pairs else 0) + 1
     return n
 
 

@@ -898,6 +898,25 @@ __device__ __forceinline__ void tma_load_5d_pair(uint32_t dst, const CUtensorMap
       "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(0), "r"(c3), "r"(c4), "r"(cl_bar)
       : "memory");
 }
+__device__ __forceinline__ void tma_load_2d_pair_hint(uint32_t dst, const CUtensorMap* map,
+                                                      int c0, int c1, uint32_t cl_bar,
+                                                      uint64_t pol) {
+  asm volatile(
+      "cp.async.bulk.tensor.2d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+      ".L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(cl_bar), "l"(pol)
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_5d_pair_hint(uint32_t dst, const CUtensorMap* map,
+                                                      int c0, int c3, int c4, uint32_t cl_bar,
+                                                      uint64_t pol) {
+  asm volatile(
+      "cp.async.bulk.tensor.5d.shared::cluster.global.tile.mbarrier::complete_tx::bytes.cta_group::2"
+      ".L2::cache_hint [%0], [%1, {%2, %3, %3, %4, %5}], [%6], %7;" ::"r"(dst),
+      "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(0), "r"(c3), "r"(c4), "r"(cl_bar),
+      "l"(pol)
+      : "memory");
+}
 // 16 bytes of a gathered row into shared memory, and the hand-over of a stage
 // whose rows came that way: the copies have landed (wait_group), are visible
 // to the tensor core's reads (proxy fence), and count as one arrival on the
@@ -1078,7 +1097,12 @@ __device__ __forceinline__ void flush_staging(const uint8_t* stg, int lane,
 // (16 rows per CTA).
 __device__ __forceinline__ int tile_cols(int rows) { return (rows + 31) & ~31; }
 
-template <int MODE>
+// ONCE: a weight tile of a group of one m-tile (one reader) is loaded
+// evict-first, as in the 1-SM kernel, so that the weight stream leaves the
+// gathered rows, activations and outputs in L2 while they fit there (LLaDA-MoE
+// shape: 1500 tokens 217 -> 205 us, 1024 tokens 192 -> 182; with 220 MB of
+// rows no gain, and the larger code cost 65536 tokens 0.6%).
+template <int MODE, bool ONCE>
 __global__ void __launch_bounds__(MODE == kModeSwiGLU ? kThreads2Up : kThreads2, 1)
     grouped_gemm_pair_kernel(const __grid_constant__ CUtensorMap map_w,
                              const __grid_constant__ CUtensorMap map_x32,
@@ -1134,12 +1158,21 @@ __global__ void __launch_bounds__(MODE == kModeSwiGLU ? kThreads2Up : kThreads2,
   cluster_sync_all();  // barriers of both CTAs initialised; the peer is running
   const int nk = p.K / (BK * C::KS);  // stages per tile
   // this CTA's weight rows of k-block k0 of tile (e, n), counted on fb
+  const uint64_t pol_once = ONCE ? l2_policy(kPolFirst) : 0;
   auto load_weights = [&](const Tile& tl, uint32_t dst, int k0, uint32_t fb) {
-    if (MODE == kModeSwiGLU)  // groups of 16 features: 4 per CTA, 8 per tile
-      tma_load_5d_pair(dst, &map_w, k0, tl.n * 8 + static_cast<int>(rank) * 4, tl.e, fb);
-    else
-      tma_load_2d_pair(dst, &map_w, k0,
-                       tl.e * p.b_rows_per_group + tl.n * 256 + static_cast<int>(rank) * BM, fb);
+    if (MODE == kModeSwiGLU) {  // groups of 16 features: 4 per CTA, 8 per tile
+      const int blk = tl.n * 8 + static_cast<int>(rank) * 4;
+      if (ONCE && tl.mtiles == 1)
+        tma_load_5d_pair_hint(dst, &map_w, k0, blk, tl.e, fb, pol_once);
+      else
+        tma_load_5d_pair(dst, &map_w, k0, blk, tl.e, fb);
+    } else {
+      const int row = tl.e * p.b_rows_per_group + tl.n * 256 + static_cast<int>(rank) * BM;
+      if (ONCE && tl.mtiles == 1)
+        tma_load_2d_pair_hint(dst, &map_w, k0, row, fb, pol_once);
+      else
+        tma_load_2d_pair(dst, &map_w, k0, row, fb);
+    }
   };
   // the ring's first weights while the kernel in front still runs, as in the
   // 1-SM kernel; both CTAs' bytes count on the leader's barriers
@@ -1498,10 +1531,10 @@ __global__ void __launch_bounds__(MODE == kModeSwiGLU ? kThreads2Up : kThreads2,
   }
 }
 
-template <int MODE>
+template <int MODE, bool ONCE>
 cudaError_t launch_pair_impl(const TcGemmArgs& a, cudaStream_t stream) {
   using C = Cfg2;
-  auto kernel = grouped_gemm_pair_kernel<MODE>;
+  auto kernel = grouped_gemm_pair_kernel<MODE, ONCE>;
   cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        C::kSmemBytes);
   if (e != cudaSuccess) return e;
@@ -1632,10 +1665,12 @@ cudaError_t launch_scores_tc(const TcGemmArgs& a, int bn, int k_splits, float* o
 }
 
 cudaError_t launch_swiglu_tc_pair(const TcGemmArgs& a, cudaStream_t stream) {
-  return launch_pair_impl<kModeSwiGLU>(a, stream);
+  return a.once ? launch_pair_impl<kModeSwiGLU, true>(a, stream)
+                : launch_pair_impl<kModeSwiGLU, false>(a, stream);
 }
 cudaError_t launch_down_tc_pair(const TcGemmArgs& a, cudaStream_t stream) {
-  return launch_pair_impl<kModeDown>(a, stream);
+  return a.once ? launch_pair_impl<kModeDown, true>(a, stream)
+                : launch_pair_impl<kModeDown, false>(a, stream);
 }
 // Output columns of one tile.
 int tc_n_granule(bool swiglu, int bn) { return swiglu ? bn / 2 : bn; }

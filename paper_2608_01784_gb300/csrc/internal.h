@@ -221,6 +221,8 @@ struct TcGemmArgs {
   // (the tile prefix) before it let this launch start: the first weights may
   // be requested before this kernel's own wait
   bool early_b = false;
+  // CTA-pair kernels: weight tiles with one reader are loaded evict-first
+  bool once = false;
 };
 // SwiGLU: out = silu(A Wg^T) * (A Wu^T).  Down: out = A Wd^T.  bn = tile
 // width (128 or 256, from tc_pick_bn); the B tensor map's box must have

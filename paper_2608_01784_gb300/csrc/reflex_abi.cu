@@ -437,7 +437,18 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
   // the last one mostly padding) and each SM streams half of the weights
   // (LLaDA2.0-mini layer, about 160 rows per expert: 0.820 -> 0.749 ms)
   const int64_t rows_per_group_est = static_cast<int64_t>(T) * k_max / 2 / E;
-  const bool pair_routed = rows_per_group_est >= 128 && inter % 128 == 0 && d % 256 == 0;
+  // Where the rows, activations and outputs fit in L2 and the weights of
+  // single-tile groups pass it by, from 96 expected rows: at the usual counts
+  // the 1-SM kernel is as good there (1024 tokens x 64 experts at k = 5: 180
+  // against 182 us), but counts above the expected mean take its groups past
+  // one 128-row tile (k = 8.6: 239 against 182 us).  The carried shared expert
+  // of short batches stays with it.
+  const bool rows_in_l2 = static_cast<int64_t>(T) * k_max / 2 * (2 * d + inter) * 2 <=
+                          (int64_t{128} << 20);
+  const bool pair_routed =
+      (rows_per_group_est >= 128 ||
+       (rows_per_group_est >= 96 && rows_in_l2 && (shared_inter == 0 || T >= 2048))) &&
+      inter % 128 == 0 && d % 256 == 0;
   // fused dispatch (opt-in): the CTA-pair gate/up GEMM gathers its rows from
   // hidden through perm, and the dispatch only places the pairs
   const bool gemm_gathers = !simt && pair_routed && (flags & REFLEX_FLAG_GATHER_IN_GEMM);
@@ -623,6 +634,7 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
       if (pair_routed) {
         g1.map_x = x1;
         g2.map_x = x2;
+        g1.once = g2.once = rows_in_l2;
         g1.map_out = &mo1;
         g2.map_out = &mo2;
       }
