@@ -136,8 +136,9 @@ __device__ __forceinline__ int group_of_tile(const GroupRows& g, int mt) {
 // MODE 0: act = silu(x Wg^T) * (x Wu^T), BN / 2 columns per tile (the first
 // half of the B tile holds gate rows, the second the matching up rows);
 // MODE 1: y = x W^T, BN columns per tile.  x [rows, K], w rows of length K.
-template <typename Te, typename C, int MODE>
-__global__ void __launch_bounds__(C::NT, 1)
+// PER_SM: CTAs per SM that the registers allow.
+template <typename Te, typename C, int MODE, int PER_SM>
+__global__ void __launch_bounds__(C::NT, PER_SM)
     gemm_simt_kernel(const Te* __restrict__ x, const Te* __restrict__ w, int K, int n_total,
                      GroupRows g, Te* __restrict__ out) {
   constexpr int TM = C::TM, TN = C::TN, BM = C::BM, BN = C::BN, BK = C::BK, HN = TN / 2;
@@ -349,7 +350,104 @@ __global__ void __launch_bounds__(C::NT, 1)
   }
 }
 
-template <typename Te, typename C, int MODE>
+// One or two rows per expert: the weights are the work, each row of them read
+// for a row or two, and one warp per output row and column streams them best
+// (16 tokens, 32 experts of 512, d = 1024: 126 us, 141 with 16-row tiles).
+// The warp's lanes split the reduction index in 8-element vectors and a
+// butterfly adds the 32 partials.
+constexpr int kDotRows = 8;   // one warp per row
+constexpr int kDotCols = 16;  // columns per CTA (loop inside the warp)
+
+__device__ __forceinline__ int group_of(const GroupRows& g, int r) {
+  if (g.offsets == nullptr) return 0;
+  int lo = 0, hi = g.E;  // offsets[lo] <= r < offsets[hi]
+  while (hi - lo > 1) {
+    const int mid = (lo + hi) >> 1;
+    if (g.offsets[mid] <= r) lo = mid; else hi = mid;
+  }
+  return lo;
+}
+
+__device__ __forceinline__ int rows_of(const GroupRows& g) {
+  if (g.offsets == nullptr) return g.dense_rows;
+  const int n = g.totals[0];
+  return n < g.cap_rows ? n : g.cap_rows;
+}
+
+__device__ __forceinline__ float warp_sum(float v) {
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+  return v;
+}
+
+template <typename Te>
+__global__ void __launch_bounds__(kDotRows * 32)
+    swiglu_dot_kernel(const Te* __restrict__ x, const Te* __restrict__ wgu,
+                       int d, int inter, GroupRows g, Te* __restrict__ act) {
+  grid_dep_wait();
+  grid_dep_launch();
+  const int lane = threadIdx.x & 31;
+  const int r = blockIdx.x * kDotRows + (threadIdx.x >> 5);
+  if (r >= rows_of(g)) return;
+  const int e = group_of(g, r);
+  const Te* xr = x + static_cast<int64_t>(r) * d;
+  const Te* wg_e = wgu + static_cast<int64_t>(e) * 2 * inter * d;
+  for (int cc = 0; cc < kDotCols; ++cc) {
+    const int c = blockIdx.y * kDotCols + cc;
+    if (c >= inter) break;
+    const Te* wg = wg_e + static_cast<int64_t>(c) * d;
+    const Te* wu = wg_e + static_cast<int64_t>(inter + c) * d;
+    float ga = 0.f, ua = 0.f;
+    for (int k = lane * 8; k < d; k += 256) {
+      float xv[8], gv[8], uv[8];
+      load8(xr + k, xv);
+      load8(wg + k, gv);
+      load8(wu + k, uv);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        ga = __fmaf_rn(xv[i], gv[i], ga);
+        ua = __fmaf_rn(xv[i], uv[i], ua);
+      }
+    }
+    ga = warp_sum(ga);
+    ua = warp_sum(ua);
+    if (lane == 0) {
+      const float s = ga / (1.0f + expf(-ga));
+      act[static_cast<int64_t>(r) * inter + c] = from_f32<Te>(s * ua);
+    }
+  }
+}
+
+template <typename Te>
+__global__ void __launch_bounds__(kDotRows * 32)
+    down_dot_kernel(const Te* __restrict__ act, const Te* __restrict__ wd,
+                     int d, int inter, GroupRows g, Te* __restrict__ y) {
+  grid_dep_wait();
+  grid_dep_launch();
+  const int lane = threadIdx.x & 31;
+  const int r = blockIdx.x * kDotRows + (threadIdx.x >> 5);
+  if (r >= rows_of(g)) return;
+  const int e = group_of(g, r);
+  const Te* ar = act + static_cast<int64_t>(r) * inter;
+  const Te* wd_e = wd + static_cast<int64_t>(e) * d * inter;
+  for (int nn = 0; nn < kDotCols; ++nn) {
+    const int n = blockIdx.y * kDotCols + nn;
+    if (n >= d) break;
+    const Te* wrow = wd_e + static_cast<int64_t>(n) * inter;
+    float acc = 0.f;
+    for (int c = lane * 8; c < inter; c += 256) {
+      float av[8], wv[8];
+      load8(ar + c, av);
+      load8(wrow + c, wv);
+#pragma unroll
+      for (int i = 0; i < 8; ++i) acc = __fmaf_rn(av[i], wv[i], acc);
+    }
+    acc = warp_sum(acc);
+    if (lane == 0) y[static_cast<int64_t>(r) * d + n] = from_f32<Te>(acc);
+  }
+}
+
+template <typename Te, typename C, int MODE, int PER_SM>
 cudaError_t launch_tile(const Te* x, const Te* w, int K, int n_total, const GroupRows& g,
                         Te* out, cudaStream_t stream) {
   const int cols = MODE == 0 ? C::BN / 2 : C::BN;
@@ -357,25 +455,47 @@ cudaError_t launch_tile(const Te* x, const Te* w, int K, int n_total, const Grou
                          ? (static_cast<int64_t>(g.cap_rows) + kTileM - 1) / kTileM + g.E
                          : (static_cast<int64_t>(g.dense_rows) + kTileM - 1) / kTileM;
   const dim3 grid(static_cast<unsigned>(mt * (kTileM / C::BM)), (n_total + cols - 1) / cols);
-  return launch_pdl(gemm_simt_kernel<Te, C, MODE>, grid, dim3(C::NT), 0, stream, x, w, K,
+  return launch_pdl(gemm_simt_kernel<Te, C, MODE, PER_SM>, grid, dim3(C::NT), 0, stream, x, w, K,
                     n_total, g, out);
 }
 
 template <typename Te, int MODE>
 cudaError_t launch_mode(const void* x, const void* w, int K, int n_total, const GroupRows& g,
                         void* out, int num_sms, cudaStream_t stream) {
-  // Large tiles once the expected pairs (half of the row capacity) fill the
-  // SMs with them; below that the small tiles' extra CTAs win.
+  // Large tiles once the expected pairs (half of the row capacity) fill half
+  // of one per group and the SMs with them; below that the small tiles' extra
+  // CTAs and fewer padding rows win (48 tokens, 32 experts of 512, d = 1024:
+  // 247 us with large tiles, 155 with small).  Small tiles run two CTAs per
+  // SM when there are more than the SMs take at a time (200 tokens, 16 experts
+  // of 512, d = 1024: 180 -> 151 us), else one with twice the registers (tiny
+  // layer 35 -> 30 us).
   const int64_t groups = g.offsets != nullptr ? g.E : 1;
   const int64_t rows = (g.offsets != nullptr ? g.cap_rows / 2 : g.dense_rows) / groups;
-  const int cols = MODE == 0 ? TileLarge::BN / 2 : TileLarge::BN;
-  const int64_t tiles =
-      groups * ((rows + TileLarge::BM - 1) / TileLarge::BM) * ((n_total + cols - 1) / cols);
+  auto tiles = [&](int bm, int cols) {
+    return groups * ((rows + bm - 1) / bm > 0 ? (rows + bm - 1) / bm : 1) *
+           ((n_total + cols - 1) / cols);
+  };
+  constexpr int kDiv = MODE == 0 ? 2 : 1;  // output columns of a tile: BN / kDiv
   const Te* xt = static_cast<const Te*>(x);
   const Te* wt = static_cast<const Te*>(w);
-  if (tiles >= num_sms)
-    return launch_tile<Te, TileLarge, MODE>(xt, wt, K, n_total, g, static_cast<Te*>(out), stream);
-  return launch_tile<Te, TileSmall, MODE>(xt, wt, K, n_total, g, static_cast<Te*>(out), stream);
+  Te* ot = static_cast<Te*>(out);
+  // fewer than two expected rows per group of many (24 tokens, 32 experts of
+  // 512, d = 1024: 143 us against 148 with 16-row tiles, 32 tokens 152 each)
+  if (g.offsets != nullptr && g.cap_rows < 4 * groups &&
+      tiles(TileSmall::BM, TileSmall::BN / kDiv) > num_sms) {
+    const dim3 grid((g.cap_rows + kDotRows - 1) / kDotRows, (n_total + kDotCols - 1) / kDotCols);
+    if constexpr (MODE == 0)
+      return launch_pdl(swiglu_dot_kernel<Te>, grid, dim3(kDotRows * 32), 0, stream, xt, wt, K,
+                        n_total, g, ot);
+    else
+      return launch_pdl(down_dot_kernel<Te>, grid, dim3(kDotRows * 32), 0, stream, xt, wt, n_total,
+                        K, g, ot);
+  }
+  if (rows >= TileLarge::BM / 2 && tiles(TileLarge::BM, TileLarge::BN / kDiv) >= num_sms)
+    return launch_tile<Te, TileLarge, MODE, 1>(xt, wt, K, n_total, g, ot, stream);
+  if (tiles(TileSmall::BM, TileSmall::BN / kDiv) > num_sms)
+    return launch_tile<Te, TileSmall, MODE, 2>(xt, wt, K, n_total, g, ot, stream);
+  return launch_tile<Te, TileSmall, MODE, 1>(xt, wt, K, n_total, g, ot, stream);
 }
 
 int max_rows(const GroupRows& g) {

@@ -30,6 +30,8 @@ def _case(dtype, T, E, kmax, d, inter, shared, seed):
     (65, 1, 1, 320, 64, 0),
     (129, 3, 2, 192, 64, 64),     # a second 128-row group tile of one row
     (128, 1, 1, 64, 128, 0),
+    (20, 40, 2, 256, 320, 0),     # about one row per expert: warp-per-dot kernels
+    (700, 20, 2, 128, 256, 0),    # small tiles, two CTAs per SM
     (2500, 1, 1, 64, 512, 0),     # large tiles: 64 x 128
     (1999, 5, 4, 192, 320, 0),    # ragged groups, partial column tiles
     (2048, 1, 1, 1024, 640, 64),  # 32 chunks of 32 products
