@@ -481,24 +481,20 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
     zero.word = ac->err;
     zero.sum = ac->k_sum;
   }
-  // bf16 with renormalised weights, many experts and many scores: tensor-
-  // core scores screen the experts and only those that could be selected get
-  // the canonical chain (router.cu).  The recheck costs about as much per
-  // chain as 40 chains of the dense score kernels and has a latency floor, so
-  // it pays from 128 experts and 2048 x 256 scores on (LLaDA2.0-mini layer:
-  // routing 213 -> 113 us at 8192 tokens, layer 4.90 -> 4.35 ms at 65536;
-  // below 2048 tokens, and with 64 experts at every size, the dense kernels
-  // are faster).
+  // bf16 with renormalised weights, more than 256 experts and many scores:
+  // tensor-core scores screen the experts and only those that could be
+  // selected get the canonical chain, one warp per token (router.cu).  The
+  // recheck costs about as much per chain as 40 chains of the dense score
+  // kernels and has a latency floor, so it pays from 2048 x 256 scores on.
   // the score rules' counts need every score from the chain: no screen
   const bool rule = ac != nullptr && ac->a.count_rule != REFLEX_RULE_REFLEX;
   const bool screen = dtype == REFLEX_DTYPE_BF16 && (flags & REFLEX_FLAG_RENORM_TOPK) &&
                       !(flags & REFLEX_FLAG_EXACT_SCORES) && d % 128 == 0 && E >= 128 &&
                       static_cast<int64_t>(T) * E >= 2048 * 256 && !rule;
-  // the same screen batched, for up to 256 experts and many tokens: the
-  // score GEMM also sums the squares of the token rows, and the recheck
-  // streams a block of token rows and every expert row through shared
-  // memory, one chain per candidate pair (router.cu); it takes precedence
-  // over the per-token recheck (LLaDA2.0-mini layer 0.573 -> 0.546 ms)
+  // the same screen batched, for up to 256 experts: the score GEMM also sums
+  // the squares of the token rows, and the recheck streams a block of token
+  // rows and every expert row through shared memory, one chain per candidate
+  // pair (router.cu)
   const bool batch_screen = dtype == REFLEX_DTYPE_BF16 && (flags & REFLEX_FLAG_RENORM_TOPK) &&
                             !(flags & REFLEX_FLAG_EXACT_SCORES) && !rule &&
                             E <= kBatchScreenMaxExperts && d % 64 == 0 &&

@@ -229,8 +229,7 @@ def _screen_bound(layer, d, k_splits_max=16):
 
 # screened routing (tensor-core scores, exact recomputation of the experts
 # that could be selected): ids, alpha and the selected scores bit for bit
-# (the screen runs from 128 experts and 2048 x 256 scores on; up to 256
-# experts the batched recheck, above it the per-token recheck)
+# (up to 256 experts the batched recheck, above it the per-token recheck)
 @pytest.mark.parametrize("T,E,d,kmax", [
     (4096, 128, 2048, 12),   # 128-wide score tiles
     (2100, 256, 1024, 12),   # ragged token tiles, two score tiles per row
@@ -400,10 +399,11 @@ def test_screened_routing_router_rows_16_byte_aligned(T, E):
     np.testing.assert_allclose(rec["alpha"][valid], alpha[valid], rtol=G.ALPHA_RTOL, atol=1e-7)
 
 
-# The batched screen (bf16, renormalised weights; up to 64 experts from 8192
-# tokens, 65-256 experts from 2048): tensor-core scores with the token norms
-# from the same GEMM, one exact chain per candidate pair in a block of 32
-# tokens (16 above 64 experts); ids, weights and selected scores bit for bit
+# The batched screen (bf16, renormalised weights; up to 256 experts by the
+# number of scores, so the smallest expert counts here run the dense kernels):
+# tensor-core scores with the token norms from the same GEMM, one exact chain
+# per candidate pair in a block of 32 tokens (up to 64 above 64 experts); ids,
+# weights and selected scores bit for bit
 @pytest.mark.parametrize("T,E,d,kmax", [
     (8192, 64, 2048, 12),    # whole token tiles
     (9000, 64, 1024, 8),     # ragged last tile
@@ -446,7 +446,7 @@ def test_batch_screened_routing_bit_exact(T, E, d, kmax):
 @pytest.mark.parametrize("kind,E,T", [
     ("ties", 64, 8192), ("all_candidates", 64, 8192), ("cancel", 64, 8192),
     ("wide", 64, 8192),
-    # above 64 experts (16-token blocks): more candidate pairs per block
+    # above 64 experts (blocks of up to 64 tokens): more candidate pairs per block
     # than one pass of the chain loop, every expert row streamed again
     ("all_candidates", 256, 8192), ("ties", 256, 8192),
     ("all_candidates", 200, 16400), ("cancel", 256, 16384),
