@@ -57,9 +57,9 @@ METRIC = ("MoE-layer tokens/s and expert TFLOP/s (frac of roofline) REFLEX vs "
 # kernel source it was taken on; once the source differs the line reports
 # null (the counters no longer describe the kernel that ran).
 NCU_TRAFFIC = {
-    "llada_moe": (561207296, "f1ace3cfdb36717b"),
-    "llada2_mini": (1280278784, "f1ace3cfdb36717b"),
-    "llada_moe_stack16": (1634616064, "f1ace3cfdb36717b"),
+    "llada_moe": (561230336, "9c3600195b6d4e7e"),
+    "llada2_mini": (1281813248, "9c3600195b6d4e7e"),
+    "llada_moe_stack16": (1634354432, "9c3600195b6d4e7e"),
 }
 KERNEL_SOURCE = os.path.join(ROOT, "paper_2608_01784_gb300", "csrc", "experts_tc.cu")
 
