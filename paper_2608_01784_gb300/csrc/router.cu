@@ -1282,19 +1282,35 @@ __device__ __forceinline__ void chain8(float& acc, const uint4& a, const uint4& 
   fma_lo(acc, a.w, b.w);
   fma_hi(acc, a.w, b.w);
 }
+// Half width of the interval around the estimate v that holds every score the
+// chain can give, from the two row norms; +inf where there is none: an
+// estimate that is not finite, a norm that is not (a sum of squares past the
+// fp32 range, an infinity or a NaN in a row), or a product of norms so large
+// that the chain or the tensor cores may overflow on the way to a finite sum.
+__device__ __forceinline__ float screen_half_width(float v, float nh, float nw, float g) {
+  const float p = nh * nw;  // >= sum_k |h_k w_k|
+  if (!(p < 0x1p126f) || !(fabsf(v) < INFINITY)) return INFINITY;
+  return g * p * (1.0f + 0x1p-16f) + fabsf(v) * 0x1p-22f;
+}
+// The ends of that interval: without one, every score.
+__device__ __forceinline__ float screen_low(float v, float half) {
+  return half < INFINITY ? v - half : -INFINITY;
+}
+__device__ __forceinline__ float screen_high(float v, float half) {
+  return half < INFINITY ? v + half : INFINITY;
+}
 // 32-bit screening key for at most 2^B experts: the order bits of an
 // interval's lower end with the low B bits replaced by 2^B - 1 - e (so no
 // two experts tie, and the lower index wins among equal truncated values).
 // Truncation is monotone, so the k-th largest key's value part is the
 // truncated k-th largest lower end: the threshold it gives is never above
 // the exact one and the candidates are a superset of the exact candidates.
-// 0 stays free for "removed" (only a negative NaN could map there).
+// v is not a NaN, so no key is 0, which stays free for "removed".
 template <int B>
 __device__ __forceinline__ uint32_t screen_key(float v, int e) {
   constexpr uint32_t m = (1u << B) - 1u;
   v = (v == 0.0f) ? 0.0f : v;
-  const uint32_t k = (order_bits(v) & ~m) | (m - static_cast<uint32_t>(e));
-  return k != 0u ? k : 1u;
+  return (order_bits(v) & ~m) | (m - static_cast<uint32_t>(e));
 }
 
 template <int NPL>
@@ -1371,9 +1387,9 @@ __global__ void __launch_bounds__(BatchCfg<NPL>::kThreads, BatchCfg<NPL>::kMinCt
           key[i][j] = 0u;
           if (e < E) {
             const float v = zv[i][j];
-            const float del = g * nh * nwj[j] * (1.0f + 0x1p-16f) + fabsf(v) * 0x1p-22f;
-            hi[i][j] = v + del;
-            key[i][j] = screen_key<Cf::kIdBits>(v - del, e);
+            const float half = screen_half_width(v, nh, nwj[j], g);
+            hi[i][j] = screen_high(v, half);
+            key[i][j] = screen_key<Cf::kIdBits>(screen_low(v, half), e);
           }
         }
         best[i] = 0u;
@@ -1398,11 +1414,15 @@ __global__ void __launch_bounds__(BatchCfg<NPL>::kThreads, BatchCfg<NPL>::kMinCt
       for (int i = 0; i < kGroup; ++i) {
         const int tl = g0 + i * kW;
         if (tl >= Cf::kT) break;
+        // -inf with its low bits cleared reads as a NaN: with fewer than k_t
+        // intervals nothing is out, so the test is for what is surely below L
+        // (a token always keeps k_t candidates, which the selection counts on)
         const float L = from_order_bits(best[i] & ~kIdMask);
         int c = 0;
 #pragma unroll
         for (int j = 0; j < NPL; ++j) {
-          const uint32_t m = __ballot_sync(0xffffffffu, tl < nt && hi[i][j] >= L);
+          const uint32_t m = __ballot_sync(
+              0xffffffffu, tl < nt && lane + 32 * j < E && !(hi[i][j] < L));
           if (lane == 0) sm.mask[tl][j] = m;
           c += __popc(m);
         }
