@@ -998,6 +998,24 @@ __device__ __forceinline__ unsigned long long score_key(float v, int e) {
          static_cast<unsigned long long>(0xffffffffu - static_cast<uint32_t>(e));
 }
 
+// Half width of the interval around the estimate v that holds every score the
+// chain can give, from the two row norms; +inf where there is none: an
+// estimate that is not finite, a norm that is not (a sum of squares past the
+// fp32 range, an infinity or a NaN in a row), or a product of norms so large
+// that the chain or the tensor cores may overflow on the way to a finite sum.
+__device__ __forceinline__ float screen_half_width(float v, float nh, float nw, float g) {
+  const float p = nh * nw;  // >= sum_k |h_k w_k|
+  if (!(p < 0x1p126f) || !(fabsf(v) < INFINITY)) return INFINITY;
+  return g * p * (1.0f + 0x1p-16f) + fabsf(v) * 0x1p-22f;
+}
+// The ends of that interval: without one, every score.
+__device__ __forceinline__ float screen_low(float v, float half) {
+  return half < INFINITY ? v - half : -INFINITY;
+}
+__device__ __forceinline__ float screen_high(float v, float half) {
+  return half < INFINITY ? v + half : INFINITY;
+}
+
 template <int NPL>
 __global__ void __launch_bounds__(kScreenWarps * 32)
     screen_select_kernel(const __nv_bfloat16* __restrict__ h,
@@ -1053,10 +1071,10 @@ __global__ void __launch_bounds__(kScreenWarps * 32)
     if (e < E) {
       float v = zt[e];
       for (int s = 1; s < k_splits; ++s) v += zt[s * split_stride + e];
-      const float del = g * nh * nw[e] * (1.0f + 0x1p-16f) + fabsf(v) * 0x1p-22f;
+      const float half = screen_half_width(v, nh, nw[e], g);
       zs[i] = v;
-      hi[i] = v + del;
-      key[i] = score_key(v - del, e);
+      hi[i] = screen_high(v, half);
+      key[i] = score_key(screen_low(v, half), e);
     }
   }
   unsigned long long best = 0ull;
@@ -1081,7 +1099,7 @@ __global__ void __launch_bounds__(kScreenWarps * 32)
   int m = 0;
 #pragma unroll
   for (int i = 0; i < NPL; ++i) {
-    const bool c = hi[i] >= L;
+    const bool c = lane + 32 * i < E && hi[i] >= L;  // L = -inf: every expert
     const uint32_t mask = __ballot_sync(0xffffffffu, c);
     const int pos = m + __popc(mask & ((1u << lane) - 1u));
     if (c && pos < 32) s_c[wid][pos] = lane + 32 * i;
@@ -1281,23 +1299,6 @@ __device__ __forceinline__ void chain8(float& acc, const uint4& a, const uint4& 
   fma_hi(acc, a.z, b.z);
   fma_lo(acc, a.w, b.w);
   fma_hi(acc, a.w, b.w);
-}
-// Half width of the interval around the estimate v that holds every score the
-// chain can give, from the two row norms; +inf where there is none: an
-// estimate that is not finite, a norm that is not (a sum of squares past the
-// fp32 range, an infinity or a NaN in a row), or a product of norms so large
-// that the chain or the tensor cores may overflow on the way to a finite sum.
-__device__ __forceinline__ float screen_half_width(float v, float nh, float nw, float g) {
-  const float p = nh * nw;  // >= sum_k |h_k w_k|
-  if (!(p < 0x1p126f) || !(fabsf(v) < INFINITY)) return INFINITY;
-  return g * p * (1.0f + 0x1p-16f) + fabsf(v) * 0x1p-22f;
-}
-// The ends of that interval: without one, every score.
-__device__ __forceinline__ float screen_low(float v, float half) {
-  return half < INFINITY ? v - half : -INFINITY;
-}
-__device__ __forceinline__ float screen_high(float v, float half) {
-  return half < INFINITY ? v + half : INFINITY;
 }
 // 32-bit screening key for at most 2^B experts: the order bits of an
 // interval's lower end with the low B bits replaced by 2^B - 1 - e (so no

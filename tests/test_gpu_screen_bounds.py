@@ -2,7 +2,8 @@
 infinity or a NaN, rows whose sum of squares leaves the fp32 range at either
 end, router rows of the same kinds.  Ids, weights and the selected scores are
 those of REFLEX_FLAG_EXACT_SCORES bit for bit, in the batched recheck (either
-side of its two instantiations)."""
+side of its two instantiations) and in the per-token recheck (above 256
+experts)."""
 import numpy as np
 import pytest
 
@@ -44,7 +45,8 @@ TOKENS = {"overflow": lambda h: h * np.float32(1e19), "largest": lambda h: h * n
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("T,E,d", [(1025, 256, 256), (5000, 64, 256), (3100, 65, 128)])
+@pytest.mark.parametrize("T,E,d", [(1025, 256, 256), (5000, 64, 256), (3100, 65, 128),
+                                   (1800, 300, 256)])
 @pytest.mark.parametrize("router", ["finite", "overflow", "largest", "inf", "nan"])
 def test_rows_without_a_bound(T, E, d, router):
     kmax = 12
