@@ -292,11 +292,13 @@ size_t reflex_moe_workspace_size(int32_t dtype, int32_t T, int32_t d,
  *   E_e(h) = (silu(h W_g,e^T) * (h W_u,e^T)) W_d,e^T.
  * The TopK is decided on the canonical chain's scores.  bf16 layers with
  * renormalised weights screen first: tensor-core scores z~ with an interval
- * z~ -/+ (gamma_d + 2^-12 + (s+1) 2^-24) ||h_i|| ||w_e|| (gamma_d = d u /
- * (1 - d u), u = 2^-24, s split-K slices) that holds both the chain's score
- * and the exact product; experts whose interval lies below the k_i-th
+ * z~ -/+ (gamma_d + 2^-12 + (s+1) 2^-24) ||h_i|| ||w_e|| + d 2^-125 (gamma_d
+ * = d u / (1 - d u), u = 2^-24, s split-K slices) that holds both the chain's
+ * score and the exact product; experts whose interval lies below the k_i-th
  * largest lower end cannot be selected, all others are recomputed with the
- * chain.  This assumes the tensor cores' fp32 accumulation errs by at most
+ * chain.  Where a norm or an estimate is not finite, or the product of the
+ * norms is within a factor of four of the fp32 range, the interval is (-inf,
+ * inf).  This assumes the tensor cores' fp32 accumulation errs by at most
  * 2^-12 sum_k |h_k w_k|; REFLEX_FLAG_EXACT_SCORES computes every score with
  * the chain instead.
  *

@@ -895,8 +895,15 @@ cudaError_t launch_logits_res(const __nv_bfloat16* h, const __nv_bfloat16* w, in
 // recomputes every expert.
 constexpr int kScreenWarps = 8;
 
-// ||w_e||_2, rounded up (every step of the fp32 sum of squares is covered by
-// the factors below).
+// The norm of a row of d values from its fp32 sum of squares, rounded up: the
+// factors cover every rounding of the sum, the last term the squares (and
+// sums) below the smallest normal number, which lose up to half of the
+// smallest subnormal each.
+__device__ __forceinline__ float norm_up(float ss, int d) {
+  return sqrtf(ss * (1.0f + 0x1p-10f) + d * 0x1p-149f) * (1.0f + 0x1p-20f);
+}
+
+// ||w_e||_2, rounded up.
 // The first kernel of a screened forward: it also clears the zero words.
 __global__ void __launch_bounds__(256)
     wnorm_kernel(const __nv_bfloat16* __restrict__ w, int E, int d, float* __restrict__ nw,
@@ -921,7 +928,7 @@ __global__ void __launch_bounds__(256)
   }
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
-  if (lane == 0) nw[e] = sqrtf(ss * (1.0f + 0x1p-10f)) * (1.0f + 0x1p-20f);
+  if (lane == 0) nw[e] = norm_up(ss, d);
 }
 
 // canonical chain of one (token, expert) pair: fma over k = 0 .. d-1 in
@@ -1003,11 +1010,15 @@ __device__ __forceinline__ unsigned long long score_key(float v, int e) {
 // estimate that is not finite, a norm that is not (a sum of squares past the
 // fp32 range, an infinity or a NaN in a row), or a product of norms so large
 // that the chain or the tensor cores may overflow on the way to a finite sum.
-__device__ __forceinline__ float screen_half_width(float v, float nh, float nw, float g) {
+// low (screen_low_floor) covers what gradual underflow, or a flush of subnormal
+// products and partial sums, can change in either of them.
+__device__ __forceinline__ float screen_half_width(float v, float nh, float nw, float g,
+                                                   float low) {
   const float p = nh * nw;  // >= sum_k |h_k w_k|
   if (!(p < 0x1p126f) || !(fabsf(v) < INFINITY)) return INFINITY;
-  return g * p * (1.0f + 0x1p-16f) + fabsf(v) * 0x1p-22f;
+  return g * p * (1.0f + 0x1p-16f) + fabsf(v) * 0x1p-22f + low;
 }
+__device__ __forceinline__ float screen_low_floor(int d) { return d * 0x1p-125f; }
 // The ends of that interval: without one, every score.
 __device__ __forceinline__ float screen_low(float v, float half) {
   return half < INFINITY ? v - half : -INFINITY;
@@ -1057,7 +1068,7 @@ __global__ void __launch_bounds__(kScreenWarps * 32)
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);
   __syncwarp();  // the row in shared memory is visible to every lane
-  const float nh = sqrtf(ss * (1.0f + 0x1p-10f)) * (1.0f + 0x1p-20f);
+  const float nh = norm_up(ss, d);
   // screen estimates and their intervals; L = k_t-th largest lower end
   float* zt = z + static_cast<int64_t>(t) * E;
   float zs[NPL], hi[NPL];
@@ -1071,7 +1082,7 @@ __global__ void __launch_bounds__(kScreenWarps * 32)
     if (e < E) {
       float v = zt[e];
       for (int s = 1; s < k_splits; ++s) v += zt[s * split_stride + e];
-      const float half = screen_half_width(v, nh, nw[e], g);
+      const float half = screen_half_width(v, nh, nw[e], g, screen_low_floor(d));
       zs[i] = v;
       hi[i] = screen_high(v, half);
       key[i] = score_key(screen_low(v, half), e);
@@ -1380,7 +1391,7 @@ __global__ void __launch_bounds__(BatchCfg<NPL>::kThreads, BatchCfg<NPL>::kMinCt
           kt[i] = kt[i] < 1 ? 1 : kcap;
         }
         rounds = max(rounds, kt[i]);
-        const float nh = sqrtf(hs[i] * (1.0f + 0x1p-10f)) * (1.0f + 0x1p-20f);
+        const float nh = norm_up(hs[i], d);
 #pragma unroll
         for (int j = 0; j < NPL; ++j) {
           const int e = lane + 32 * j;
@@ -1388,7 +1399,7 @@ __global__ void __launch_bounds__(BatchCfg<NPL>::kThreads, BatchCfg<NPL>::kMinCt
           key[i][j] = 0u;
           if (e < E) {
             const float v = zv[i][j];
-            const float half = screen_half_width(v, nh, nwj[j], g);
+            const float half = screen_half_width(v, nh, nwj[j], g, screen_low_floor(d));
             hi[i][j] = screen_high(v, half);
             key[i][j] = screen_key<Cf::kIdBits>(screen_low(v, half), e);
           }

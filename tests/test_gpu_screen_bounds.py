@@ -63,3 +63,21 @@ def test_rows_without_a_bound(T, E, d, router):
     k = np.random.default_rng(T).integers(1, kmax + 1, T).astype(np.int32)
     k[:8] = kmax
     _same_as_exact(cfg, layer, k)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("T,E,d", [(1025, 256, 256), (5000, 64, 256), (1800, 300, 256)])
+@pytest.mark.parametrize("eh,ew", [(-80, 0), (0, -80), (-70, -60), (-100, -22)])
+def test_rows_whose_squares_underflow(T, E, d, eh, ew):
+    # scores far below the products they are summed from, of rows scaled by
+    # powers of two until their squares (and, last, the products) are subnormal
+    rng = np.random.default_rng(T + E)
+    kmax = 8
+    cfg, layer = _layer(T, E, d, kmax, seed=T)
+    x = W.bf16_bits_to_f32(W.to_bf16_bits(rng.standard_normal((T, d // 2))))
+    y = W.bf16_bits_to_f32(W.to_bf16_bits(rng.standard_normal((E, d // 2))))
+    eps = (1e-3 * rng.standard_normal((E, d // 2))).astype(np.float32)
+    h, w = np.concatenate([x, x], 1), np.concatenate([y, eps - y], 1)
+    layer["hidden"] = W.to_bf16_bits(h * np.float32(2.0 ** eh))
+    layer["w_router"] = W.to_bf16_bits(w * np.float32(2.0 ** ew))
+    _same_as_exact(cfg, layer, rng.integers(1, kmax + 1, T).astype(np.int32))
