@@ -154,8 +154,11 @@ __global__ void __launch_bounds__(C::NT, PER_SM)
     e = group_of_tile(g, mt);
     if (e < 0) return;
     const int first = g.offsets[e], last = g.offsets[e + 1];
-    row0 = first + (mt - g.mt_prefix[e]) * kTileM + sub * BM;
-    if (first < 0 || last > g.cap_rows) return;  // inconsistent workspace
+    // values of an inconsistent workspace can be any: no row outside [0, cap)
+    const int64_t at = static_cast<int64_t>(first) +
+                       (static_cast<int64_t>(mt) - g.mt_prefix[e]) * kTileM + sub * BM;
+    if (first < 0 || last > g.cap_rows || at >= last) return;
+    row0 = static_cast<int>(at);
     rows = min(BM, last - row0);
   } else {
     row0 = mt * kTileM + sub * BM;
