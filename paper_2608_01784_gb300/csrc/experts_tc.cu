@@ -330,16 +330,23 @@ __device__ __forceinline__ bool decode_tile(const KParams& p, const TileIndex& i
     const int mid = (lo + hi) >> 1;
     if (p.n_tiles * ix.pref[mid] <= t) lo = mid; else hi = mid;
   }
-  const int mt_e = ix.pref[lo + 1] - ix.pref[lo];
-  if (mt_e <= 0) return false;
-  const int l = t - p.n_tiles * ix.pref[lo];
+  // an inconsistent workspace can hold any values; in unsigned arithmetic
+  // whatever wraps fails one of the comparisons
+  const uint32_t first = ix.pref[lo], last = ix.pref[lo + 1];
+  const uint32_t row_lo = ix.offs[lo], row_hi = ix.offs[lo + 1];
+  const uint32_t mt_e = last - first, most = p.max_mtiles;
+  if (mt_e - 1u >= most) return false;
+  const uint32_t l = t - p.n_tiles * first, n = l / mt_e;
+  const uint32_t row0 = row_lo + (l - n * mt_e) * p.tile_rows;
   o.e = lo;
   o.mtiles = mt_e;
-  o.n = l / mt_e;
-  o.row0 = ix.offs[lo] + (l % mt_e) * p.tile_rows;
-  o.rows = min(p.tile_rows, ix.offs[lo + 1] - o.row0);
-  return o.n < p.n_tiles && o.row0 >= 0 && o.rows > 0 &&
-         o.row0 + o.rows <= p.g.cap_rows;
+  o.n = n;
+  o.row0 = row0;
+  o.rows = min(static_cast<uint32_t>(p.tile_rows), row_hi - row0);
+  // row_hi <= cap < 2^31 and (l mod mt_e) tile_rows < cap + E tile_rows, so
+  // row0 cannot wrap past row_lo while row_lo <= row_hi
+  return n < static_cast<uint32_t>(p.n_tiles) && row_lo <= row0 && row0 < row_hi &&
+         row_hi <= static_cast<uint32_t>(p.g.cap_rows);
 }
 
 // Expert, n-tile and m-tile count of tile t, read before the kernel's

@@ -23,6 +23,10 @@ SIMT = RENORM | B.REFLEX_FLAG_SIMT_EXPERTS
     ("f32", 2500, 2, 512, RENORM),   # 64-row tiles
     ("f32", 20, 40, 320, RENORM),    # warp-per-dot kernels
     ("bf16", 300, 4, 128, SIMT),
+    ("bf16", 300, 4, 128, RENORM),   # 1-SM tiles
+    ("bf16", 1100, 4, 128, RENORM),  # CTA-pair tiles
+    ("bf16", 1100, 4, 128, RENORM | B.REFLEX_FLAG_GATHER_IN_GEMM),
+    ("bf16", 600, 40, 128, RENORM),
 ])
 def test_expert_stages_stay_in_their_buffers(dtype, T, E, inter, flags):
     d, kmax = 256, 2
