@@ -1753,41 +1753,60 @@ cudaError_t logits_dispatch(const __nv_bfloat16* h, const __nv_bfloat16* w, int 
                             int num_sms, cudaStream_t s, const L2Prefetch& pf) {
   const int sms = num_sms > 0 ? num_sms : 1;
   const int64_t per_sm = static_cast<int64_t>(T) * E / sms;
+  // CTAs of tiles of bt x be chains per SM (rounded up)
+  auto ctas_per_sm = [&](int64_t bt, int64_t be) {
+    return ((T + bt - 1) / bt * ((E + be - 1) / be) + sms - 1) / sms;
+  };
   // Whole rows resident while every CTA of the grid is (one or two per SM, by
   // their shared memory): a chain then costs little more than its fma latency.
-  // Small tiles first, since few rows are also loaded soonest (score and
-  // selection kernels, us, against the ring kernel): 4 x 16, 32 tokens x 64
-  // experts 15.2 -> 10.6, 64 x 256 16.9 -> 12.1; 8 x 16, 512 x 64 17.6 ->
-  // 16.0; 16 x 32 of 2 x 1 chains per thread, 700 x 64 19.8 -> 18.3, 1024 x
-  // 64 scores 20.8 -> 18.1 alone.  With more CTAs than fit at a time the ring
-  // kernel's smaller tiles win (1500 x 64: 31.7 -> 25.3).
+  // Small tiles first, since few rows are also loaded soonest.  Score and
+  // selection kernels in us, d = 2048, 64 experts, against the ring kernel
+  // of the same size: 4 x 16 tiles 237 tokens 10.1 / 14.6; 8 x 16 332 tokens
+  // 14.7 / 15.2, 546 15.3 / 15.7, but 593 (two CTAs of 97 KB on nearly every
+  // SM) 17.5 / 15.7, so these stop at 7 CTAs for four SMs where only two fit
+  // one; 16 x 32 of 2 x 1 chains per thread 593 tokens 17.0 / 15.7, 641 17.0 /
+  // 18.3, 736 17.3 / 18.4: once the ring's 16 x 16 tiles need two CTAs on an
+  // SM.  With more CTAs than fit at a time the ring
+  // wins (1425 x 64: 24.2; in two rounds of resident rows 31.7).
   using R1 = ResCfg<4, 1, 1, 1, 2>;
   using R2 = ResCfg<4, 1, 1, 2, 2>;
   using R3 = ResCfg<4, 2, 1, 2, 4>;
-  auto resident = [&](int bt, int be, size_t smem, int most) {
+  auto resident = [&](int bt, int be, size_t smem, int most, int most_if_two) {
     const int64_t ctas = static_cast<int64_t>((T + bt - 1) / bt) * ((E + be - 1) / be);
     const int fit = static_cast<int>(static_cast<size_t>(227 * 1024) / (smem + 1024));
+    const int quarters = fit >= 3 ? most : fit == 2 ? most_if_two : fit * 4;
     return d % kResChunkK == 0 && d / kResChunkK <= kResMaxChunks &&
-           ctas <= static_cast<int64_t>(sms) * (fit < most ? fit : most);
+           4 * ctas <= static_cast<int64_t>(sms) * (quarters < most ? quarters : most);
   };
-  if (resident(R1::BT, R1::BE, R1::smem(d), 2))
+  if (resident(R1::BT, R1::BE, R1::smem(d), 8, 8))
     return launch_logits_res<4, 1, 1, 1, 2>(h, w, T, d, E, z, zero, err, pf, s);
-  if (resident(R2::BT, R2::BE, R2::smem(d), 2))
+  if (resident(R2::BT, R2::BE, R2::smem(d), 8, 7))
     return launch_logits_res<4, 1, 1, 2, 2>(h, w, T, d, E, z, zero, err, pf, s);
-  if (resident(R3::BT, R3::BE, R3::smem(d), 1))
+  if (ctas_per_sm(16, 16) > 1 && resident(R3::BT, R3::BE, R3::smem(d), 4, 4))
     return launch_logits_res<4, 2, 1, 2, 4>(h, w, T, d, E, z, zero, err, pf, s);
-  // Ring kernel, score and selection kernels in us: 1 x 2 against 1 x 1 tiles
-  // 512 x 64 16.2 / 17.7, 256 x 64 15.8 / 15.4; 4 x 4 tiles of two-warp CTAs
-  // while one warp per scheduler holds every chain, 4096 x 64 42.3 against
-  // 44.7 (2 x 2); 2 x 4 tiles 1536 x 256 59.2 against 63.8; 4 x 4 again 2048 x
-  // 256 67.5 against 72.6.
+  // Ring kernel: 1 x 1 tiles while one CTA of them per SM holds the chains
+  // (142 x 64 14.4 us, 1 x 2 tiles 15.0; 380 x 64 16.7 / 15.3), 1 x 2 tiles up
+  // to two CTAs of 2 x 2 per SM (2375 x 64 28.6 against 29.7; 2612 x 64 35.3
+  // each).
   if (per_sm <= 160 || E <= 8)
     return launch_logits_mx<4, 1, 1, 4, 1, 8>(h, w, T, d, E, z, zero, s);
   if (per_sm <= 1080) return launch_logits_mx<4, 1, 2, 4, 1, 8>(h, w, T, d, E, z, zero, s);
-  if (per_sm <= 1500) return launch_logits_mx<4, 2, 2, 2, 2, 4, 64>(h, w, T, d, E, z, zero, s);
-  if (per_sm > 2048 && per_sm <= 3072 && E > 32)
-    return launch_logits_mx<4, 2, 4, 2, 2, 4, 64>(h, w, T, d, E, z, zero, s);
-  if (per_sm <= 4300) return launch_logits_mx<8, 4, 4, 1, 2, 4, 64>(h, w, T, d, E, z, zero, s);
+  // Then 2 x 2 tiles (16 x 32 chains, four warps) or 4 x 4 (32 x 32, two
+  // warps).  Both take the longer the more CTAs an SM gets, in steps: n CTAs
+  // of 2 x 2 tiles, or p pairs of CTAs of 4 x 4, which together have a warp per
+  // scheduler.  A pair costs as much as 3.2 CTAs of 2 x 2 (d = 2048, us):
+  //   n       3     4     5     6     7     8     9     10    11
+  //   2 x 2   35.6  42.5  50.6  59.5  68.3  77.0  87.4  96    106
+  //   4 x 4   40.3  40.5  62.5  63.0  63.5  63.8  92.3  93    94
+  // With six, 2 x 4 tiles (16 x 64 chains) take 57.5 if no column is padding.
+  if (per_sm <= 4300) {
+    const int64_t n = ctas_per_sm(16, 32), p = (ctas_per_sm(32, 32) + 1) / 2;
+    if (10 * n > 32 * p + 3)
+      return launch_logits_mx<8, 4, 4, 1, 2, 4, 64>(h, w, T, d, E, z, zero, s);
+    if (n == 6 && (E + 63) / 64 * 2 == (E + 31) / 32)
+      return launch_logits_mx<4, 2, 4, 2, 2, 4, 64>(h, w, T, d, E, z, zero, s);
+    return launch_logits_mx<4, 2, 2, 2, 2, 4, 64>(h, w, T, d, E, z, zero, s);
+  }
   if (per_sm <= 10000) return launch_logits_mx<8, 4, 8, 2, 2, 3, 64>(h, w, T, d, E, z, zero, s);
   if (per_sm <= 20000) return launch_logits_mx<8, 4, 4, 2, 2, 3, 64>(h, w, T, d, E, z, zero, s);
   return launch_logits_mx<8, 4, 8, 2, 2, 4>(h, w, T, d, E, z, zero, s);

@@ -169,17 +169,17 @@ def _bf16_case(T, d, E, inter, shared, kmax, seed, weight_std=0.05):
 
 # every score-kernel band of the bf16 router (chains T x E per SM on 152 SMs)
 @pytest.mark.parametrize("T,E,d", [
-    (100, 64, 2048),     # ring kernel, 1 x 1 thread tiles
+    (100, 64, 2048),     # whole rows resident, 4 x 16 tiles
     (1000, 64, 2048),    # whole rows resident, ragged token tile
     (1200, 48, 512),     # whole rows resident, ragged expert tile
     (250, 256, 1024),    # whole rows resident, 4 chunks
-    (700, 128, 2048),    # whole rows resident, ragged token tile, 4 expert tiles
+    (700, 128, 2048),    # ring kernel, 1 x 2, ragged token tile
     (2000, 32, 512),     # whole rows resident, one expert tile
-    (500, 160, 1024),    # whole rows resident, 5 expert tiles, ragged expert tile
+    (500, 160, 1024),    # ring kernel, 1 x 2, ten expert tiles
     (2000, 64, 256),     # ring kernel, 1 x 2
-    (4096, 64, 256),     # ring kernel, 2 x 2, 64-k chunks
+    (4096, 64, 256),     # ring kernel, 4 x 4, two warps
     (8192, 128, 256),    # ring kernel, 4 x 8
-    (8192, 256, 256),    # ring kernel, 4 x 4
+    (8192, 256, 256),    # ring kernel, 4 x 4, four warps
     (16384, 256, 256),   # ring kernel, 4 x 8, 4 stages
 ])
 def test_router_scores_bit_exact_every_band(T, E, d):
