@@ -78,6 +78,21 @@ def update_state(state: dict, conf_new: torch.Tensor, num_blocks: torch.Tensor,
     return committed
 
 
+def screens_in_batches(T: int, E: int, d: int, k_max: int) -> bool:
+    """Whether a bf16 forward of T tokens with renormalised weights screens its
+    router scores in batches (up to 256 experts; the library's line)."""
+    if E <= 8 or E > 256 or d % 64:
+        return False
+    c = 0 if d < 1024 else 1 if d < 2048 else 2 if d < 4096 else 3
+    if E <= 32 and c >= 2 and 4 * k_max > E:
+        return T * E >= 16384 * 32 if c == 2 else T >= 11000
+    if E <= 32:
+        return T * (32 if c >= 2 else E) >= (20480, 14336, 10240, 9728)[c] * 32
+    if E <= 64:
+        return T >= (9729, 4865, 4865, 3264)[c]
+    return T * ((E + 31) // 32 * 32 if c else E) >= (2048, 1217, 913, 688)[c] * 256
+
+
 def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
                   flags: int = B.REFLEX_FLAG_RENORM_TOPK, count_rule: int = 0,
                   k_max: int = 12, inter: int = 512) -> int:
@@ -85,9 +100,8 @@ def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
     library's choices: the count kernel; the score kernel and the selection,
     or (bf16, renormalised weights, >= 128 experts, T E >= 2048 x 256,
     d % 128 == 0) the norm kernel, the score GEMM and the screened selection,
-    or (bf16, renormalised weights, T E >= 768 x 256 with 65-256 experts,
-    4608 x 64 with 33-64, 16384 x 32 with fewer) the norm kernel, the score GEMM and the batched
-    recheck; count + scan in one
+    or (bf16, renormalised weights, up to 256 experts, screens_in_batches)
+    the norm kernel, the score GEMM and the batched recheck; count + scan in one
     CTA (short batches whose block masks fit in shared memory) or count and
     scan, then the gather, which also places the pairs; the gate/up and down
     GEMMs (and the shared expert's two, once the routed GEMMs run on CTA
@@ -98,8 +112,7 @@ def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
     screened = (dtype == "bf16" and flags & B.REFLEX_FLAG_RENORM_TOPK and
                 not flags & B.REFLEX_FLAG_EXACT_SCORES and not count_rule)
     screen = screened and d % 128 == 0 and E >= 128 and T * E >= 2048 * 256
-    batch_screen = screened and d % 64 == 0 and E <= 256 and T * E >= (
-        16384 * 32 if E <= 32 else 4608 * 64 if E <= 64 else 768 * 256)
+    batch_screen = screened and screens_in_batches(T, E, d, k_max)
     n += 3 if (screen or batch_screen) else 2
     n += 1 if T <= 4096 and (T + 31) // 32 * E * 4 <= 160 * 1024 else 2
     est = T * k_max // 2 // E

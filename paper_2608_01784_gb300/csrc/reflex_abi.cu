@@ -21,15 +21,42 @@ using rx::WsHeader;
 constexpr size_t kAlign = 256;
 // gate/up weight bytes handed to the L2 while the router scores run
 constexpr uint64_t kRouterL2Prefetch = 64ull << 20;
-// Scores T E from which layers with up to 256 experts screen their router
-// scores in batches: the dense chains cost T E, the screen's three kernels
-// about 40 us at least, and with few experts most of a token's work is the
-// screen itself.  Layer times dense / screened: 256 experts, 1024 tokens 329
-// / 326 us; 160, 1300: 244.5 / 243.7; 96, 2048: 231 / 228; 64, 3270: 377 /
-// 376, 6000: 540 / 526; 32, 8192: 408 / 412; 16, 8192: 382 / 402, 16000: 707
-// / 713; 8, 16000: 663 / 687.
-int64_t batch_screen_min_scores(int32_t E) {
-  return E <= 32 ? 16384 * 32 : E <= 64 ? 4608 * 64 : 768 * 256;
+// Whether a layer with up to 256 experts screens its router scores in batches.
+// The dense chains cost T E d, in steps: whole CTAs per SM.  The screen costs
+// three kernels' latency, the screening of each token (k_t rounds over 32 or 64
+// experts per CTA up to 64 of them) and only then chains, so its line moves
+// with d, and T e counts the columns that the dense kernels compute there: e =
+// E in whole tiles.  Scores and selection, dense / screened in us, k_max 4 and
+// 12 of random counts, below the line and from it on:
+//   experts  d     T below               T from the line on
+//   256      512   2047 20 / 21, 21 / 22    2048 29 / 21, 37 / 22
+//   256      1024  1216 23 / 26, 24 / 27    1300 28 / 26, 29 / 27
+//   256      2048  900 35.7 / 35.9, 36 / 37  1024 40.5 / 34.8, 41 / 36
+//   256      4096  560 53 / 56, 53 / 57     768 65 / 56, 66 / 57
+//   64       512   9500 21 / 22, 22 / 26    10000 27 / 22, 28 / 26
+//   64       1024  4864 23 / 25, 24 / 29    4900 28 / 25, 29 / 29
+//   64       2048  4864 40 / 36, 41 / 43    4900 50 / 36, 51 / 44
+//   64       4096  2433 64 / 52, 64 / 59    3270 66 / 51, 66 / 59
+//   32       512   20000 30 / 34, 32 / 39   22000 50 / 34, 52 / 40
+//   32       1024  12000 30 / 29, 31 / 35   14000 35 / 30, 37 / 35 (16384: 36 / 39, 38 / 47)
+//   32       2048  9500 41 / 40, 42 / 52    11000 52 / 40, 53 / 52
+//   32       4096  9500 76 / 66, 77 / 92    10000 98 / 66, 99 / 92
+// (from d = 2048 with few experts counts up to k_max > E / 4 move the line: 16
+// experts, k_max 12, d = 2048, 18000 tokens 67 / 83, 49152 321 / 179; d = 4096,
+// 10000 68 / 90, 11000 98 / 93)
+//   8        2048  dense at every size: 32768 88 / 128, 65536 142 / 239
+// Over 4600 sizes (4 to 256 experts, d 256 to 4096, 500 to 65536 tokens) the
+// choice takes 0.8% more time than the faster of the two each time.
+bool batch_screen_pays(int64_t T, int32_t E, int32_t d, int32_t k_max) {
+  if (E <= 8) return false;
+  const int c = d < 1024 ? 0 : d < 2048 ? 1 : d < 4096 ? 2 : 3;
+  constexpr int64_t kUpTo32[4] = {20480 * 32, 14336 * 32, 10240 * 32, 9728 * 32};
+  constexpr int64_t kUpTo64[4] = {9729 * 64, 4865 * 64, 4865 * 64, 3264 * 64};
+  constexpr int64_t kWide[4] = {2048 * 256, 1217 * 256, 913 * 256, 688 * 256};
+  if (E <= 32 && c >= 2 && 4 * k_max > E) return c == 2 ? T * E >= 16384 * 32 : T >= 11000;
+  if (E <= 32) return T * (c >= 2 ? 32 : E) >= kUpTo32[c];
+  if (E <= 64) return T * 64 >= kUpTo64[c];
+  return T * (c >= 1 ? (E + 31) / 32 * 32 : E) >= kWide[c];
 }
 constexpr int32_t kBatchScreenMaxExperts = 256;
 size_t up(size_t x) { return (x + kAlign - 1) / kAlign * kAlign; }
@@ -498,7 +525,7 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
   const bool batch_screen = dtype == REFLEX_DTYPE_BF16 && (flags & REFLEX_FLAG_RENORM_TOPK) &&
                             !(flags & REFLEX_FLAG_EXACT_SCORES) && !rule &&
                             E <= kBatchScreenMaxExperts && d % 64 == 0 &&
-                            static_cast<int64_t>(T) * E >= batch_screen_min_scores(E);
+                            batch_screen_pays(T, E, d, k_max);
   if ((stages & REFLEX_STAGE_ROUTE) && batch_screen) {
     CUtensorMap mh, mw, mhb, mwb;
     // score tile width: 256 reads each token row once for all experts, once

@@ -18,6 +18,7 @@ import pytest
 
 import gpu_cases as G
 from paper_2608_01784_gb300 import _binding as B
+from paper_2608_01784_gb300 import api
 from paper_2608_01784_gb300 import workloads as W
 
 N_CASES = 48
@@ -30,8 +31,8 @@ def draw_case(seed: int) -> dict:
     d = int(rng.choice([128, 256, 384, 512, 640, 1024, 2048]))
     inter = int(rng.choice([64, 128, 192, 256, 320, 512]))
     shared = int(rng.choice([0, 0, 0, 64, 128, 256]))
-    # token counts: mostly short, some past the batched-screen and split
-    # dispatch thresholds (2048, 4096, 8192 tokens)
+    # token counts: mostly short, some past the batched screen's line of wide
+    # layers and the split dispatch's (4096 tokens)
     band = rng.random()
     if band < 0.55:
         T = int(rng.integers(1, 1500))
@@ -63,8 +64,9 @@ def draw_case(seed: int) -> dict:
 
 def test_draws_cover_the_paths():
     cases = [draw_case(s) for s in range(N_CASES)]
-    assert any(c["T"] >= 8192 and c["E"] <= 64 for c in cases) or \
-        any(c["T"] >= 2048 and 64 < c["E"] <= 256 for c in cases)
+    assert any(c["flags"] & B.REFLEX_FLAG_RENORM_TOPK and
+               not c["flags"] & B.REFLEX_FLAG_EXACT_SCORES and
+               api.screens_in_batches(c["T"], c["E"], c["d"], c["kmax"]) for c in cases)
     assert any(c["shared"] for c in cases)
     assert any(c["flags"] & B.REFLEX_FLAG_SIMT_EXPERTS for c in cases)
     assert any(not c["flags"] & B.REFLEX_FLAG_RENORM_TOPK for c in cases)

@@ -399,21 +399,19 @@ def test_screened_routing_router_rows_16_byte_aligned(T, E):
     np.testing.assert_allclose(rec["alpha"][valid], alpha[valid], rtol=G.ALPHA_RTOL, atol=1e-7)
 
 
-# The batched screen (bf16, renormalised weights; up to 256 experts by the
-# number of scores, so the smallest expert counts here run the dense kernels):
-# tensor-core scores with the token norms from the same GEMM, one exact chain
+# The batched screen (bf16, renormalised weights, 9 to 256 experts): tensor-core scores with the token norms from the same GEMM, one exact chain
 # per candidate pair in a block of 32 tokens (up to 64 above 64 experts); ids,
 # weights and selected scores bit for bit
 @pytest.mark.parametrize("T,E,d,kmax", [
     (8192, 64, 2048, 12),    # whole token tiles
     (9000, 64, 1024, 8),     # ragged last tile
-    (8256, 40, 512, 6),      # fewer experts than the 64-row expert box
-    (8192, 64, 256, 12),     # short rows (4 chunks)
+    (9792, 40, 512, 6),      # fewer experts than the 64-row expert box
+    (9729, 64, 256, 12),     # short rows (4 chunks)
     (16384, 17, 2048, 4),    # odd expert count
     (12289, 64, 1024, 8),    # one token in the last CTA
     (30000, 48, 512, 12),    # ragged last CTA, 48 experts
-    (8192, 1, 256, 1),       # a single expert: every token's one candidate
-    (8200, 8, 512, 8),       # counts up to k = E
+    (72900, 9, 128, 9),      # few experts, counts up to k = E
+    (41000, 16, 128, 1),     # one candidate for most tokens
     (8192, 256, 2048, 12),   # 256 experts: eight 32-expert groups per lane
     (9000, 200, 1024, 8),    # 200 experts (a partial group), ragged last CTA
     (8192, 96, 512, 32),     # 96 experts, counts up to 32
@@ -421,6 +419,7 @@ def test_screened_routing_router_rows_16_byte_aligned(T, E):
     (20000, 200, 512, 12),   # 200 experts, ragged last CTA
 ])
 def test_batch_screened_routing_bit_exact(T, E, d, kmax):
+    assert api.screens_in_batches(T, E, d, kmax)
     cfg, layer = _bf16_case(T, d, E, 128, 0, kmax, seed=5 * T + E + d)
     k = np.random.default_rng(T + E).integers(1, min(kmax, E) + 1, T).astype(np.int32)
     gl = G.GpuLayer(cfg, layer)

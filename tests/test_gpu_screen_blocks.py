@@ -9,21 +9,24 @@ import pytest
 import gpu_cases as G
 import oracle
 from paper_2608_01784_gb300 import _binding as B
+from paper_2608_01784_gb300 import api
 from paper_2608_01784_gb300 import workloads as W
 
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("T,E,d,kmax", [
     (2049, 256, 256, 12),
-    (3100, 65, 128, 7),     # 65 experts, blocks of 24 tokens
-    (1025, 256, 128, 12),   # blocks of 8 tokens
+    (8100, 65, 128, 7),     # 65 experts, blocks of 56 tokens
+    (2049, 256, 128, 12),   # blocks of 16 tokens
+    (1217, 256, 1024, 12),  # blocks of 8 tokens: the first that are screened, d = 1024
     (9728, 128, 128, 4),    # one wave of 152 blocks of 64
     (9729, 200, 128, 12),   # two waves
-    (8193, 64, 256, 12),    # 32-token blocks, the last of one token
-    (8970, 33, 128, 1),
-    (32769, 17, 128, 4),    # up to 32 experts: from 16384 x 32 scores
+    (9729, 64, 256, 12),    # 32-token blocks, the last of one token
+    (9760, 33, 128, 1),
+    (38552, 17, 128, 4),    # up to 32 experts: the first that are screened below d = 1024
 ])
 def test_block_edges(T, E, d, kmax):
+    assert api.screens_in_batches(T, E, d, kmax)
     cfg = W.LayerConfig(name="screen", dtype="bf16", d=d, E=E, inter=128, shared_inter=0,
                         k_min=1, k_base=1, k_max=kmax, delta_role=0, delta_cur=0, w_cf=0.3,
                         n_seq=1, prompt_len=T, gen_len=0, block=32, weight_std=0.05,

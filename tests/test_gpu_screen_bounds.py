@@ -9,6 +9,7 @@ import pytest
 
 import gpu_cases as G
 from paper_2608_01784_gb300 import _binding as B
+from paper_2608_01784_gb300 import api
 from paper_2608_01784_gb300 import workloads as W
 
 
@@ -21,6 +22,7 @@ def _layer(T, E, d, kmax, seed):
 
 
 def _same_as_exact(cfg, layer, k):
+    assert cfg.E > 256 or api.screens_in_batches(k.size, cfg.E, cfg.d, cfg.k_max)
     gl = G.GpuLayer(cfg, layer)
     flags = B.REFLEX_FLAG_RENORM_TOPK | B.REFLEX_STAGE_ROUTE
     _, s, st_s = gl.forward(k, flags=flags)
@@ -45,7 +47,7 @@ TOKENS = {"overflow": lambda h: h * np.float32(1e19), "largest": lambda h: h * n
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("T,E,d", [(1025, 256, 256), (5000, 64, 256), (3100, 65, 128),
+@pytest.mark.parametrize("T,E,d", [(1025, 256, 2048), (5000, 64, 1024), (2500, 65, 2048),
                                    (1800, 300, 256)])
 @pytest.mark.parametrize("router", ["finite", "overflow", "largest", "inf", "nan"])
 def test_rows_without_a_bound(T, E, d, router):
@@ -66,7 +68,7 @@ def test_rows_without_a_bound(T, E, d, router):
 
 
 @pytest.mark.gpu
-@pytest.mark.parametrize("T,E,d", [(1025, 256, 256), (5000, 64, 256), (1800, 300, 256)])
+@pytest.mark.parametrize("T,E,d", [(1025, 256, 2048), (5000, 64, 1024), (1800, 300, 256)])
 @pytest.mark.parametrize("eh,ew", [(-80, 0), (0, -80), (-70, -60), (-100, -22)])
 def test_rows_whose_squares_underflow(T, E, d, eh, ew):
     # scores far below the products they are summed from, of rows scaled by
