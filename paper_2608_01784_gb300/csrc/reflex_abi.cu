@@ -583,14 +583,14 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
     // kernel before the router reads it
     // the first experts' gate/up weights are handed to the L2 while the
     // scores run (the grouped GEMM walks the experts in order; LLaDA-MoE
-    // layer step -2 us with 64 MB), once the expected pairs (T k_max / 2) are
-    // six per expert: below that the prefetch brings experts that nobody
-    // needs and delays the short score kernel's own loads (layer with /
-    // without, LLaDA-MoE shape: 100 tokens 152.7 / 154.4 us, 32 tokens 156.6 /
-    // 153.3; LLaDA2.0-mini shape: 16 tokens 135.8 / 133.0, 1 token 69 / 55)
+    // layer step -2 us with 64 MB), from 24 tokens: fewer need too few of
+    // those experts, and their few CTAs pass on little (layer without / with:
+    // 64 experts of 1024, d = 2048, 8 tokens 74.5 / 74.8 us, 16 109.0 / 107.7,
+    // 32 127.4 / 125.8, 100 147.5 / 143.2; 256 of 512, 8 tokens 60.6 / 60.7, 24
+    // 107.9 / 104.9, 200 260.2 / 253.5; 128 of 1024, d = 1024, 8 tokens 55.0 /
+    // 55.2, 24 90.3 / 89.9, 64 126.5 / 124.3)
     rx::L2Prefetch pf;
-    if ((stages & REFLEX_STAGE_EXPERT_UP) &&
-        static_cast<int64_t>(T) * k_max >= 12 * static_cast<int64_t>(E)) {
+    if ((stages & REFLEX_STAGE_EXPERT_UP) && T >= 24) {
       const uint64_t wbytes =
           static_cast<uint64_t>(E) * 2 * inter * d * (dtype == REFLEX_DTYPE_F32 ? 4 : 2);
       pf.base = w_gate_up;
