@@ -116,7 +116,7 @@ def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
     n += 3 if (screen or batch_screen) else 2
     n += 1 if T <= 4096 and (T + 31) // 32 * E * 4 <= 160 * 1024 else 2
     est = T * k_max // 2 // E
-    pairs = est >= 128 or (est >= 96 and d <= 2048 and T >= 2048 and
+    pairs = est >= 128 or (est >= (96 if d <= 2048 else 104 if E >= 32 else 128) and T >= 2048 and
                            T * k_max // 2 * (2 * d + inter) * 2 <= 128 << 20)
     n += 1 + 2 + (2 if shared_inter and pairs else 0) + 1
     return n

@@ -466,10 +466,10 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
   const int64_t rows_per_group_est = static_cast<int64_t>(T) * k_max / 2 / E;
   // Where the rows, activations and outputs fit in L2 and the weights of
   // single-tile groups pass it by, from 96 expected rows (k_max / 2 a token)
-  // up to d = 2048.  The 1-SM kernel is as good or slightly better while no
-  // group passes one 128-row tile, and takes up to a third longer as soon as
-  // some do, so the line lies where the counts that callers use (k_base, or a
-  // mean of k_max / 2) balance.  Layer, CTA pairs against 1-SM, mean over 13
+  // up to d = 2048, more above.  The 1-SM kernel is as good or slightly better
+  // while no group passes one 128-row tile, and takes up to a third longer as
+  // soon as some do, so the line lies where the counts that callers use
+  // (k_base, or a mean of k_max / 2) balance.  Layer, CTA pairs against 1-SM, mean over 13
   // shapes of 8 to 128 experts, 512 to 2048 wide, d = 2048, at 4, 5, 6, 1..12
   // and 8 experts a token (k_max 12; 88 rows: three shapes, 3 instead of 4):
   //    88 rows  +1.1%  +2.1%  +1.6%   +2.0%   -3.7%
@@ -478,14 +478,17 @@ static int forward_impl(int32_t dtype, const void* hidden, const void* w_router,
   //   112       +0.7   +0.5   -1.1    -5.9   -21.4
   //   127       +0.2   -0.9   -14.3   -16.2  -21.5
   // d = 1024 is alike (96: +0.6, +1.2, +0.1, +0.2, -10.6).  At d = 4096 pairs
-  // take 7 to 8% longer until groups pass a tile (96: +7.0, +7.8, +8.4, +2.7,
-  // -3.0; 104: +7.2, +7.6, +8.2, +0.9, -13.5), so those keep the line at 128.
+  // take 5 to 11% longer until groups pass a tile, most with few experts, whose
+  // weight tiles are few: the line is 104 from 32 experts on and 128 below (32
+  // to 64 experts, 96 rows: +5.7, +6.1, +6.4, +2.7, -8.4; 104: +5.7, +5.9, +6.0,
+  // +0.0, -19.0; 8 and 16, 112: +8.0, +8.9, +9.9, +2.1, -11.0; 127: +10.2, +11.0,
+  // -3.1, -6.6, -9.1).
   // The carried shared expert of short batches stays with the 1-SM kernel.
   const bool rows_in_l2 = static_cast<int64_t>(T) * k_max / 2 * (2 * d + inter) * 2 <=
                           (int64_t{128} << 20);
   const bool pair_routed =
       (rows_per_group_est >= 128 ||
-       (rows_per_group_est >= 96 && d <= 2048 && rows_in_l2 &&
+       (rows_per_group_est >= (d <= 2048 ? 96 : E >= 32 ? 104 : 128) && rows_in_l2 &&
         (shared_inter == 0 || T >= 2048))) &&
       inter % 128 == 0 && d % 256 == 0;
   // fused dispatch (opt-in): the CTA-pair gate/up GEMM gathers its rows from
