@@ -1789,9 +1789,13 @@ cudaError_t logits_dispatch(const __nv_bfloat16* h, const __nv_bfloat16* w, int 
   };
   if (resident(R1::BT, R1::BE, R1::smem(d), 8, 8))
     return launch_logits_res<4, 1, 1, 1, 2>(h, w, T, d, E, z, zero, err, pf, s);
-  if (resident(R2::BT, R2::BE, R2::smem(d), 8, 7))
+  // With weights to prefetch the whole band stays: the ring kernel does not
+  // prefetch, which costs the layer more than its scores gain (560 tokens x
+  // 64 experts of 512: 100.5 us, 103.7 with the ring).
+  const bool prefetch = pf.bytes > 0;
+  if (resident(R2::BT, R2::BE, R2::smem(d), 8, prefetch ? 8 : 7))
     return launch_logits_res<4, 1, 1, 2, 2>(h, w, T, d, E, z, zero, err, pf, s);
-  if (ctas_per_sm(16, 16) > 1 && resident(R3::BT, R3::BE, R3::smem(d), 4, 4))
+  if ((prefetch || ctas_per_sm(16, 16) > 1) && resident(R3::BT, R3::BE, R3::smem(d), 4, 4))
     return launch_logits_res<4, 2, 1, 2, 4>(h, w, T, d, E, z, zero, err, pf, s);
   // Ring kernel: 1 x 1 tiles while one CTA of them per SM holds the chains
   // (142 x 64 14.4 us, 1 x 2 tiles 15.0; 380 x 64 16.7 / 15.3), 1 x 2 tiles up
