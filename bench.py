@@ -489,7 +489,7 @@ def run_gpu(args, cfg, rank, world, local_rank):
         layer_bytes += 3 * S * d * es
     layer_flops = flops_step + (6.0 * d * S * T if S else 0.0)
     t_roof = max(layer_bytes / (peaks["hbm"] * 1e9), layer_flops / (peaks["bf16"] * 1e12))
-    launches_per_step = api.step_launches(cfg.dtype, T, d, E, S, F)
+    launches_per_step = api.step_launches(cfg.dtype, T, d, E, S, F, k_max=cfg.k_max, inter=I)
     line = dict(
         metric=METRIC, value=tokens_per_s, unit="tokens/s",
         n_gpus=world, steps=args.steps, warmup=args.warmup, ms_per_step=ms_step,
@@ -842,7 +842,8 @@ def run_stack(args, rank, world, local_rank):
                 frac_of_burst=tf / peaks["bf16"],
                 peak_source=peaks["source"] + " (sustained bf16; the kernel runs "
                                               "inside a long step)")
-    launches = 1 + L * (api.step_launches(cfg.dtype, T, d, E, 0, F) - 1)
+    launches = 1 + L * (api.step_launches(cfg.dtype, T, d, E, 0, F, k_max=cfg.k_max,
+                                             inter=cfg.inter) - 1)
     line = dict(
         metric=METRIC, value=R.whole_job_rate(T, world, ms_step), unit="tokens/s",
         n_gpus=world, steps=args.steps, warmup=args.warmup, ms_per_step=ms_step,

@@ -78,6 +78,9 @@ def update_state(state: dict, conf_new: torch.Tensor, num_blocks: torch.Tensor,
     return committed
 
 
+_NUM_SMS = 152  # of the GPU that the library is built for
+
+
 def screens_in_batches(T: int, E: int, d: int, k_max: int) -> bool:
     """Whether a bf16 forward of T tokens with renormalised weights screens its
     router scores in batches (up to 256 experts; the library's line)."""
@@ -104,8 +107,8 @@ def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
     the norm kernel, the score GEMM and the batched recheck; count + scan in one
     CTA (short batches whose block masks fit in shared memory) or count and
     scan, then the gather, which also places the pairs; the gate/up and down
-    GEMMs (and the shared expert's two, once the routed GEMMs run on CTA
-    pairs; the 1-SM launches carry its tiles); the combine.
+    GEMMs (and the shared expert's two, unless the routed GEMMs run on single
+    SMs in tiles that divide its width, and carry it); the combine.
     With a score count rule the selection derives the counts: no count
     kernel and no screen.  Memsets are not kernels."""
     n = 0 if count_rule else 1
@@ -115,11 +118,20 @@ def step_launches(dtype: str, T: int, d: int, E: int, shared_inter: int,
     batch_screen = screened and screens_in_batches(T, E, d, k_max)
     n += 3 if (screen or batch_screen) else 2
     n += 1 if T <= 4096 and (T + 31) // 32 * E * 4 <= 160 * 1024 else 2
+    n += 1 + 2 + 1
+    if not shared_inter:
+        return n
+    if dtype != "bf16" or flags & B.REFLEX_FLAG_SIMT_EXPERTS:
+        return n + 2
     est = T * k_max // 2 // E
-    pairs = est >= 128 or (est >= (96 if d <= 2048 else 104 if E >= 32 else 128) and T >= 2048 and
-                           T * k_max // 2 * (2 * d + inter) * 2 <= 128 << 20)
-    n += 1 + 2 + (2 if shared_inter and pairs else 0) + 1
-    return n
+    rows_in_l2 = T * k_max // 2 * (2 * d + inter) * 2 <= 128 << 20
+    line = 96 if d <= 2048 else 104 if E >= 32 else 128
+    pairs = inter % 128 == 0 and d % 256 == 0 and (
+        est >= 128 or (est >= line and rows_in_l2 and T >= 2048))
+    # 1-SM tiles: 256 wide (128 gate/up columns) once they fill the SMs 8 times over
+    m_tiles = E + (T * k_max // 2 + 127) // 128
+    cols = 128 if inter % 128 == 0 and inter // 128 * m_tiles >= 8 * _NUM_SMS else 64
+    return n if not pairs and shared_inter % cols == 0 else n + 2
 
 
 class MoELayer:

@@ -193,4 +193,40 @@ def test_step_launch_count_matches_a_profile(name):
              if e.device_type == torch.autograd.DeviceType.CUDA and "rx::" in e.name]
     if not names:
         pytest.skip("no kernel activity recorded by the profiler")
-    assert len(names) == api.step_launches(cfg.dtype, cfg.T, cfg.d, cfg.E, cfg.shared_inter)
+    assert len(names) == api.step_launches(cfg.dtype, cfg.T, cfg.d, cfg.E, cfg.shared_inter,
+                                           k_max=cfg.k_max, inter=cfg.inter)
+
+
+@pytest.mark.parametrize("dtype,T,E,d,inter,shared,kmax", [
+    ("bf16", 300, 512, 256, 512, 128, 4),   # 256-wide tiles carry the shared expert
+    ("bf16", 300, 512, 256, 512, 64, 4),    # ... or do not divide its width
+    ("bf16", 2048, 8, 256, 128, 128, 2),    # CTA pairs: its own launches
+    ("bf16", 2048, 8, 256, 192, 128, 2),    # 192 columns: no CTA pairs
+    ("bf16", 2048, 8, 384, 128, 128, 2),    # d of no whole 256 columns
+    ("bf16", 2100, 16, 256, 128, 128, 2),   # 131 expected rows
+    ("bf16", 1200, 256, 1024, 128, 0, 12),  # dense scores, then screened
+    ("bf16", 1217, 256, 1024, 128, 0, 12),
+    ("f32", 100, 8, 256, 128, 128, 2),
+])
+def test_step_launch_count_over_the_choices(dtype, T, E, d, inter, shared, kmax):
+    profiler = pytest.importorskip("torch.profiler")
+    cfg = W.CONFIGS["llada_moe"].with_(
+        name="launches", dtype=dtype, d=d, E=E, inter=inter, shared_inter=shared, k_min=1,
+        k_base=min(2, kmax), k_max=kmax, delta_role=0, delta_cur=0, n_seq=1, prompt_len=T - 32,
+        gen_len=32, weight_std=0.05)
+    dl = api.layer_to_device(W.make_layer(cfg, 1), cfg.dtype)
+    moe = api.MoELayer(dl, dtype=dtype, d=d, E=E, inter=inter, shared_inter=shared, k_max=kmax,
+                       max_tokens=T)
+    p = G.params_of(cfg)
+    ds = api.state_to_device(W.make_state(cfg, 0))
+    moe.step(ds, p, dl["hidden"])
+    torch.cuda.synchronize()
+    for _ in range(2):  # the first warms the profiler itself
+        with profiler.profile(activities=[profiler.ProfilerActivity.CUDA]) as prof:
+            moe.step(ds, p, dl["hidden"])
+            torch.cuda.synchronize()
+    names = [e.name for e in prof.events()
+             if e.device_type == torch.autograd.DeviceType.CUDA and "rx::" in e.name]
+    if not names:
+        pytest.skip("no kernel activity recorded by the profiler")
+    assert len(names) == api.step_launches(dtype, T, d, E, shared, k_max=kmax, inter=inter), names
