@@ -231,3 +231,18 @@ def test_default_params_count_rule_is_reflex(lib):
     lib.reflex_default_params(ctypes.byref(p))
     assert p.count_rule == B.REFLEX_RULE_REFLEX and p.rule_threshold == 0.0
     assert ctypes.sizeof(B.reflex_alloc_params) == 64
+
+
+def test_current_stream_without_the_private_entry(monkeypatch):
+    # the stream handle comes from torch's public Stream where the private
+    # entry for the handle alone is missing
+    import torch
+    from paper_2608_01784_gb300 import _binding as B
+
+    class Current:
+        cuda_stream = 1234
+
+    monkeypatch.delattr(torch._C, "_cuda_getCurrentRawStream", raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda: Current)
+    monkeypatch.setattr(torch.cuda, "current_device", lambda: 0)
+    assert B._stream(None) == 1234
