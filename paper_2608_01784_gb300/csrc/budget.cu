@@ -70,9 +70,9 @@ __device__ __forceinline__ int clip(int k, int lo, int hi) {
   return k < lo ? lo : (k > hi ? hi : k);
 }
 
-// The counts of sequence s; its error bits and the sum of its counts go to
-// err_bits and sum of thread 0.
-__device__ __forceinline__ void budget_body(int s, const float* __restrict__ conf1,
+// The counts of the block's sequence; its error bits and the sum of its counts
+// go to err_bits and sum of thread 0.
+__device__ __forceinline__ void budget_body(const float* __restrict__ conf1,
                                             const float* __restrict__ conf2,
                                             const uint8_t* __restrict__ hist_len,
                                             const uint8_t* __restrict__ masked,
@@ -90,6 +90,7 @@ __device__ __forceinline__ void budget_body(int s, const float* __restrict__ con
   __shared__ int s_nj;
   __shared__ unsigned long long s_sum;
   __shared__ uint32_t s_err;
+  const int s = blockIdx.x;
   const int lo = seq_off[s], hi = seq_off[s + 1];
   if (lo < 0 || hi > T || lo > hi) {  // malformed offsets: touch no count
     err_bits = kErrIndex;
@@ -212,7 +213,6 @@ __device__ __forceinline__ void budget_body(int s, const float* __restrict__ con
   __syncthreads();
   err_bits = s_err;
   sum = s_sum;
-  __syncthreads();  // the shared words before the next sequence's
 }
 
 // defer = 0: waits for the previous kernel before reading anything.
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(kThreads)
   grid_dep_launch();
   uint32_t bits;
   unsigned long long sum;
-  budget_body(blockIdx.x, conf1, conf2, hist_len, masked, block_id, seq_off, active_block, T, a,
+  budget_body(conf1, conf2, hist_len, masked, block_id, seq_off, active_block, T, a,
               k_out, bits, sum);
   if (defer) grid_dep_wait();
   if (threadIdx.x == 0) {
