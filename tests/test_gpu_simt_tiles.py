@@ -6,6 +6,7 @@ and bf16 layer tolerances (a dot product of K terms errs by at most
 K 2^-24 sum |x w|; 32-term chunks keep it far below)."""
 import numpy as np
 import pytest
+import torch
 
 import gpu_cases as G
 from paper_2608_01784_gb300 import _binding as B
@@ -67,3 +68,61 @@ def test_an_overflowing_sum_stays_infinite(T, inter):
     out, _, status = gl.forward(np.ones(T, np.int32))
     assert status == B.REFLEX_OK
     assert np.all(np.isposinf(out))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("T,inter", [(40, 64), (2500, 512)])
+def test_rows_without_finite_sums_leave_the_others_alone(T, inter):
+    # up weights of 1e38: rows of ones overflow to +inf (as above), rows of
+    # 1e-3 do not; a NaN in a row makes its outputs NaN
+    d = 64
+    cfg, layer = _case("f32", T, 1, 1, d, inter, 0, seed=T)
+    h = layer["hidden"].reshape(T, d)
+    h[:] = np.float32(1e-3) * (1 + np.arange(T, dtype=np.float32)[:, None] / T)
+    layer["w_gate_up"][:, :inter] = 1.0
+    layer["w_gate_up"][:, inter:] = 1e38
+    layer["w_down"][:] = 1e-3
+    clean, _, status = G.GpuLayer(cfg, layer).forward(np.ones(T, np.int32))
+    assert status == B.REFLEX_OK and np.all(np.isfinite(clean))
+    big, nan = np.arange(0, T, 9), np.arange(4, T, 9)
+    h[big] = 1.0
+    h[nan, 7] = np.nan
+    out, _, status = G.GpuLayer(cfg, layer).forward(np.ones(T, np.int32))
+    assert status == B.REFLEX_OK
+    assert np.all(np.isposinf(out[big])) and np.all(np.isnan(out[nan]))
+    rest = np.setdiff1d(np.arange(T), np.concatenate([big, nan]))
+    assert np.array_equal(out[rest].view(np.uint32), clean[rest].view(np.uint32))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("where", ["rows", "weights"])
+def test_values_without_finite_sums_cost_little(where):
+    # 14 times the layer's time for a NaN in every row and 6.5 times for an
+    # infinity in a gate row of every expert (all outputs NaN or infinite)
+    # where single threads summed the outputs again; 1.1 and 3.8 with warps
+    T, E, d, inter = 1024, 16, 1024, 512
+    cfg, layer = _case("f32", T, E, 2, d, inter, 0, seed=3)
+    gl = G.GpuLayer(cfg, layer)
+    k = torch.full((T,), 2, dtype=torch.int32, device="cuda")
+    out = torch.empty_like(gl.dev["hidden"])
+
+    def us():
+        a, b = (torch.cuda.Event(enable_timing=True) for _ in range(2))
+        best = 1e9
+        for _ in range(4):
+            a.record()
+            for _ in range(10):
+                gl.moe.forward(gl.dev["hidden"], k, out)
+            b.record()
+            torch.cuda.synchronize()
+            best = min(best, a.elapsed_time(b) * 100)
+        return best
+
+    clean = us()
+    if where == "rows":
+        gl.dev["hidden"][:, 3] = float("nan")
+    else:
+        gl.moe.w["w_gate_up"][:, 7, 5] = float("inf")
+    bad = us()
+    assert gl.moe.status() == B.REFLEX_OK and not bool(torch.isfinite(out).any())
+    assert bad <= (2.0 if where == "rows" else 5.0) * clean, (clean, bad)
