@@ -412,9 +412,8 @@ __global__ void __launch_bounds__(C::NT, PER_SM)
   }
 }
 
-// One or two rows per expert: the weights are the work, each row of them read
-// for a row or two, and one warp per output row and column streams them best
-// (16 tokens, 32 experts of 512, d = 1024: 126 us, 141 with 16-row tiles).
+// A few rows per expert: the weights are the work, each row of them read for
+// these rows, and one warp per output row and column streams them best.
 // The warp's lanes split the reduction index in 8-element vectors and a
 // butterfly adds the 32 partials.
 constexpr int kDotRows = 8;   // one warp per row
@@ -541,10 +540,22 @@ cudaError_t launch_mode(const void* x, const void* w, int K, int n_total, const 
   const Te* xt = static_cast<const Te*>(x);
   const Te* wt = static_cast<const Te*>(w);
   Te* ot = static_cast<Te*>(out);
-  // fewer than two expected rows per group of many (24 tokens, 32 experts of
-  // 512, d = 1024: 143 us against 148 with 16-row tiles, 32 tokens 152 each)
-  if (g.offsets != nullptr && g.cap_rows < 4 * groups &&
-      tiles(TileSmall::BM, TileSmall::BN / kDiv) > num_sms) {
+  // A few expected rows per group of enough weights: the dot kernels.  fp32 below
+  // two rows, where the small tiles are more than the SMs; bf16, half of whose
+  // weight bytes make the dots that much cheaper while the tiles' cost stays, up
+  // to six, from 2^20 weights of a projection on.  Layer, dot kernels against
+  // tiles, mean over 24 to 40 shapes (4 to 128 experts, d 256 to 2048, 128 to
+  // 512 wide), with as many rows as expected and with twice as many:
+  //   fp32, many tiles   1.5 rows -22%, -13%   2 -18, -3   2.5 -13, +9   3 -6, +26
+  //   bf16, many tiles   4 rows -32%, -4%   5 -27, +9   6 -15, +26   8 -3, +25
+  //   bf16, few tiles    4 rows -7, -1   5 -3, +3 (2^19 weights +5, 2^18 +22)   6 -1, +8
+  // (at two rows and a little above, fp32 tiles round 3% less off).
+  const bool dots = sizeof(Te) == 2
+                        ? g.cap_rows <= 12 * groups &&
+                              groups * n_total * static_cast<int64_t>(K) >= (1 << 20)
+                        : g.cap_rows < 4 * groups &&
+                              tiles(TileSmall::BM, TileSmall::BN / kDiv) > num_sms;
+  if (g.offsets != nullptr && dots) {
     const dim3 grid((g.cap_rows + kDotRows - 1) / kDotRows, (n_total + kDotCols - 1) / kDotCols);
     if constexpr (MODE == 0)
       return launch_pdl(swiglu_dot_kernel<Te>, grid, dim3(kDotRows * 32), 0, stream, xt, wt, K,

@@ -32,6 +32,10 @@ def _case(dtype, T, E, kmax, d, inter, shared, seed):
     (129, 3, 2, 192, 64, 64),     # a second 128-row group tile of one row
     (128, 1, 1, 64, 128, 0),
     (20, 40, 2, 256, 320, 0),     # about one row per expert: warp-per-dot kernels
+    (96, 32, 4, 128, 256, 0),     # six expected rows: the last for bf16's dot kernels
+    (97, 32, 4, 128, 256, 0),
+    (31, 32, 4, 256, 512, 0),     # below two expected rows: the last for fp32's
+    (32, 32, 4, 256, 512, 0),
     (700, 20, 2, 128, 256, 0),    # small tiles, two CTAs per SM
     (2500, 1, 1, 64, 512, 0),     # large tiles: 64 x 128
     (1999, 5, 4, 192, 320, 0),    # ragged groups, partial column tiles
