@@ -749,12 +749,16 @@ __device__ __forceinline__ void mx_fma8(float (&acc)[TM][TN], const MxOps<TM, TN
   }
 }
 
-// What one CTA can hand on while it computes its scores (about 10 us): more
-// of it makes the kernel wait for the TMA unit.  Layer in us with 0, 256, 512,
-// 1024, 2048 KB per CTA and without a bound: 16 tokens x 8 experts of 1024, d =
-// 2048, 43.9, 44.0, 44.2, 45.7, 49.7, 109.2; 33 x 32, 1024, 94.4, 94.5, 93.4,
-// 93.7, 97.4, 103.6; 100 x 64, 1024, 147.8, 144.8, 143.5, 143.3, 143.4, 143.6.
-constexpr uint64_t kL2PrefetchPerCta = 512 * 1024;
+// What one CTA can hand on while it computes its scores (about 10 us at d =
+// 2048): more of it makes the kernel wait for the TMA unit.  Layer in us with 0,
+// 256, 512, 1024, 2048 KB per CTA and without a bound: 16 tokens x 8 experts of
+// 1024, d = 2048, 43.9, 44.0, 44.2, 45.7, 49.7, 109.2; 33 x 32, 1024, 94.4, 94.5,
+// 93.4, 93.7, 97.4, 103.6; 100 x 64, 1024, 147.8, 144.8, 143.5, 143.3, 143.4,
+// 143.6.  Short rows leave less time: 24 tokens x 16 experts of 128, d = 256, 24.3
+// with none, 25.4 with 512 KB, 24.7 with 128.
+constexpr uint64_t l2_prefetch_per_cta(int d) {
+  return 512 * static_cast<uint64_t>(d < 1024 ? d : 1024);
+}
 // Each CTA hands its share of [pf.base, pf.base + pf.bytes) to the L2 as
 // bulk prefetches (the TMA unit moves them; no thread waits for them).
 __device__ __forceinline__ void l2_prefetch_share(const L2Prefetch& pf) {
@@ -878,7 +882,7 @@ cudaError_t launch_logits_res(const __nv_bfloat16* h, const __nv_bfloat16* w, in
   if (e != cudaSuccess) return e;
   const dim3 g((T + C::BT - 1) / C::BT, (E + C::BE - 1) / C::BE);
   L2Prefetch share = pf;
-  const uint64_t most = static_cast<uint64_t>(g.x) * g.y * kL2PrefetchPerCta;
+  const uint64_t most = static_cast<uint64_t>(g.x) * g.y * l2_prefetch_per_cta(d);
   if (share.bytes > most) share.bytes = most;
   kern<<<g, C::NT, smem, s>>>(h, w, T, d, E, z, zero, err, share);
   return cudaGetLastError();
