@@ -1,9 +1,11 @@
 """The SIMT expert GEMMs at the edges of their tiles (16 x 64 and 64 x 128
-outputs, k blocks of 64 and 16, 128-row group tiles), against the oracle:
+outputs, k blocks of 64 and 32, 128-row group tiles), against the oracle:
 one row, one row either side of a tile, column counts that leave a partial
-last tile, and both tile sizes of the dispatch.  The tolerances are the fp32
-and bf16 layer tolerances (a dot product of K terms errs by at most
-K 2^-24 sum |x w|; 32-term chunks keep it far below)."""
+last tile (64 of the 128 columns of a large down tile: every other tile width
+divides the widths that the layer takes), both tile sizes of the dispatch and
+the dot kernels.  The tolerances are the fp32 and bf16 layer tolerances (a dot
+product of K terms errs by at most K 2^-24 sum |x w|; running sums of 8 or 16
+products and their carried rounding keep it far below)."""
 import numpy as np
 import pytest
 import torch
@@ -38,8 +40,10 @@ def _case(dtype, T, E, kmax, d, inter, shared, seed):
     (32, 32, 4, 256, 512, 0),
     (700, 20, 2, 128, 256, 0),    # small tiles, two CTAs per SM
     (2500, 1, 1, 64, 512, 0),     # large tiles: 64 x 128
-    (1999, 5, 4, 192, 320, 0),    # ragged groups, partial column tiles
-    (2048, 1, 1, 1024, 640, 64),  # 32 chunks of 32 products
+    (1999, 5, 4, 192, 320, 0),    # ragged groups, small tiles
+    (4000, 5, 4, 192, 64, 0),     # large down tiles, the last of 64 columns
+    (5200, 4, 1, 320, 64, 64),    # the same in the dense shared expert
+    (2048, 1, 1, 1024, 640, 64),  # 32 k blocks
 ])
 def test_tile_edges(dtype, T, E, kmax, d, inter, shared):
     cfg, layer = _case(dtype, T, E, kmax, d, inter, shared, seed=T + d)
