@@ -71,9 +71,11 @@ extern "C" {
  * bits either way (the screen's bound is stated with reflex_moe_forward);
  * only the record's other scores differ (tensor-core estimates). */
 #define REFLEX_FLAG_EXACT_SCORES 0x8u
-/* bf16 tcgen05 path, routed gate/up GEMM on CTA pairs (at least 128 rows
- * per expert expected: T * k_max / (2 E) >= 128, inter % 128 == 0, d % 256
- * == 0): the GEMM fetches its input rows from hidden itself through the pair
+/* bf16 tcgen05 path, routed gate/up GEMM on CTA pairs (inter % 128 == 0, d %
+ * 256 == 0, and expected rows per expert, T * k_max / (2 E), of at least 128;
+ * fewer do, from 96, or 104 with d > 2048 and E >= 32, where the expected rows,
+ * activations and outputs fit in 128 MB and no shared expert is given or T >=
+ * 2048): the GEMM fetches its input rows from hidden itself through the pair
  * permutation, and DISPATCH only places the pairs (no copy of the rows in
  * pair order is written).  The outputs are the same bits as without the flag.
  * Elsewhere the flag changes nothing.  The fused dispatch is slower on GB300

@@ -100,8 +100,8 @@ inline int64_t screen_z_rows(int T, int E, int d) {
 // tensor-core estimates [T, E] (one K slice), hss the tokens' sums of
 // squares, nw the experts' norms (wnorm_kernel); map_h / map_w are 2D maps of
 // the hidden states [T, d] and the router weights [E, d] with boxes of 64
-// columns and screen_batch_token_rows(E) / screen_batch_expert_rows(E) rows (128-byte
-// swizzle).  Writes ids / alpha and the candidates' exact scores into z.
+// columns and screen_batch_token_rows(E) / screen_batch_expert_rows(E) rows, not
+// swizzled.  Writes ids / alpha and the candidates' exact scores into z.
 // the box heights of map_h (tokens per CTA) and map_w for E experts
 int screen_batch_token_rows(int E);
 int screen_batch_expert_rows(int E);

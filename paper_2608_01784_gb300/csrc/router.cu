@@ -1251,7 +1251,7 @@ struct BatchCfg {
   static constexpr int kCap = 2048;
   static constexpr uint32_t kTokBytes = kT * 128;
   static constexpr uint32_t kStageBytes = kTokBytes + kE * 128;
-  static_assert(kT % 8 == 0 && kT <= 64, "whole swizzle atoms; the prefix's 64 lanes");
+  static_assert(kT % 8 == 0 && kT <= 64, "tpc counts eights; the prefix's 64 lanes");
   static_assert(kCap >= kE, "a round holds at least one token");
 };
 template <int NPL>
