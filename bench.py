@@ -57,9 +57,9 @@ METRIC = ("MoE-layer tokens/s and expert TFLOP/s (frac of roofline) REFLEX vs "
 # kernel source it was taken on; once the source differs the line reports
 # null (the counters no longer describe the kernel that ran).
 NCU_TRAFFIC = {
-    "llada_moe": (561230336, "9c3600195b6d4e7e"),
-    "llada2_mini": (1281813248, "9c3600195b6d4e7e"),
-    "llada_moe_stack16": (1634354432, "9c3600195b6d4e7e"),
+    "llada_moe": (561020416, "22d823c163a454bc"),
+    "llada2_mini": (1281585920, "22d823c163a454bc"),
+    "llada_moe_stack16": (1634407936, "22d823c163a454bc"),
 }
 KERNEL_SOURCE = os.path.join(ROOT, "paper_2608_01784_gb300", "csrc", "experts_tc.cu")
 
