@@ -151,10 +151,10 @@ def _stream(stream) -> int | None:
         # the handle alone: building torch's Stream object takes 2.9 us, more
         # than a kernel launch (the entry is private, so not every torch need
         # have it)
-        raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
-        if raw is None:
+        try:
+            return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+        except AttributeError:
             return torch.cuda.current_stream().cuda_stream
-        return raw(torch.cuda.current_device())
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream

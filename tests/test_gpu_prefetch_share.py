@@ -52,5 +52,6 @@ def test_a_short_batch_is_no_slower_than_its_stages(T, E, d, inter):
     times = [(us(whole), us(parts)) for _ in range(7)][1:]
     best = [min(t) for t in zip(*times)]
     assert moe.status() == B.REFLEX_OK
-    # separate calls wait for each other's end; 2.2 times their time without a bound on the share
-    assert best[0] <= 1.1 * best[1], best
+    # about equal (separate calls wait for each other's end); 1.5 to 2.4 times as
+    # long without a bound on the share
+    assert best[0] <= 1.25 * best[1], best
